@@ -615,11 +615,19 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
     timing->n = 0;
     HF_CUDA(cudaEventRecord(timing->ev[timing->n++], st));
   }
-  // heaviest classes first.  The f/g (Rys) classes are many and often
-  // small: without per-class timing they fork onto the side streams (round
-  // robin) and run beside each other and the s/p/d classes; every class
-  // shares only the J/K atomics with the others.
-  bool forked = false;
+  // Heaviest classes first.  Without per-class timing the launches fork onto
+  // the side streams (round robin) and run beside each other: a class of a
+  // small molecule leaves most SMs idle while its longest items finish, and
+  // the classes share only the J/K atomics.  A build of one launch (one
+  // shell type) stays on the main stream.
+  int nlaunch = 0;
+  for (int c = 0; c < HF_NCLASS; ++c) nlaunch += (b->work64[c].w.nitems > 0) + (b->work32[c].w.nitems > 0);
+  const bool fork = !timing && nlaunch > 1;
+  const int nuse = std::min(nlaunch, (int)hf_ctx::kSide);
+  if (fork) {
+    HF_CUDA(cudaEventRecord(ctx->fork_ev, st));
+    for (int k = 0; k < nuse; ++k) HF_CUDA(cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
+  }
   int nside = 0;
   for (int c = HF_NCLASS - 1; c >= 0; --c) {
     const EriClassOps& op = ctx->ops[c];
@@ -633,15 +641,7 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
       const int occ = r == 0 ? hf_occ_hi(op, o.flags) : hf_occ_lo(op, o.flags);
       const LaunchShape sh = hf_launch_shape(ctx, occ, w.nitems);
       NvtxRange nv_cls(op.name);
-      cudaStream_t ls = st;
-      if (!timing && (op.rys_native || (o.flags & HF_JK_RYS))) {
-        if (!forked) {
-          HF_CUDA(cudaEventRecord(ctx->fork_ev, st));
-          for (int k = 0; k < hf_ctx::kSide; ++k) HF_CUDA(cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
-          forked = true;
-        }
-        ls = ctx->side[nside++ % hf_ctx::kSide];
-      }
+      const cudaStream_t ls = fork ? ctx->side[nside++ % nuse] : st;
       fn(w, ps, kc, one, nullptr, sh.grid, sh.threads, ls);
       if (timing) {
         timing->which[timing->n - 1] = 2 * c + r;
@@ -650,8 +650,8 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
     }
   }
   HF_CUDA(cudaGetLastError());
-  if (forked)
-    for (int k = 0; k < hf_ctx::kSide; ++k) {
+  if (fork)
+    for (int k = 0; k < nuse; ++k) {
       HF_CUDA(cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
       HF_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[k], 0));
     }

@@ -1208,6 +1208,11 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<hfgen::CLS, R>, 128, 0);      \
     return n;                                                                                            \
   }                                                                                                      \
+  template <typename R>                                                                                  \
+  static int occR_##CLS() { /* asked once: the same answer for every launch of the process */           \
+    static const int n = occR_query_##CLS<R>();                                                          \
+    return n;                                                                                            \
+  }                                                                                                      \
   static void launch_jk64_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const MolJK& one, \
                                 const MolJK* mols, int grid, int threads, cudaStream_t s) {              \
     launch_jkR_##CLS<double>(w, ps, kc, one, mols, grid, threads, s);                                    \
@@ -1235,9 +1240,16 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
       n = occR_##CLS<double>();                                                                          \
     return n;                                                                                            \
   }                                                                                                      \
+  static int occ_jkdf_##CLS() {                                                                          \
+    static const int n = occ_jkdf_query_##CLS();                                                         \
+    return n;                                                                                            \
+  }                                                                                                      \
   static void launch_store_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc, double* G,   \
                                  int nbf, int grid, cudaStream_t s) {                                    \
-    hfk::eri_store_kernel<hfgen::CLS><<<grid, 128, 0, s>>>(w, ps, kc, G, nbf);                           \
+    if constexpr (hfgen::CLS::COOP)                                                                      \
+      hfk::store_coop_launch<hfgen::CLS>(w, ps, kc, G, nbf, grid, s);                                    \
+    else                                                                                                 \
+      hfk::eri_store_kernel<hfgen::CLS><<<grid, 128, 0, s>>>(w, ps, kc, G, nbf);                         \
   }                                                                                                      \
   static void launch_schwarz_##CLS(const int* pairs, int npairs, const PairSet& ps, const KernelCommon& kc, \
                                    double* Q, cudaStream_t s) {                                          \

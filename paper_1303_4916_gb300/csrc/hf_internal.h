@@ -43,8 +43,8 @@ struct hf_ctx {
   float* boysdf = nullptr;
   double* rys = nullptr;    // Rys roots and weights table (rys.cuh)
   EriClassOps ops[HF_NCLASS] = {};
-  static constexpr int kSide = 4;
-  cudaStream_t side[kSide] = {};     // class launches fork onto these (multi-molecule J/K)
+  static constexpr int kSide = 8;
+  cudaStream_t side[kSide] = {};     // class launches fork onto these
   cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {};
   std::atomic<int> fail_countdown{0};
   std::atomic<long long> device_bytes{0};

@@ -1061,14 +1061,17 @@ void jk_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const
 
 template <int CLS>
 int jk_occ() {
-  static const RysClass rc = rys_class_of(CLS);
-  int n = 0;
+  static const int occ = [] {
+    const RysClass rc = rys_class_of(CLS);
+    int n = 0;
 #define RYS_O(KM)          \
   set_smem_attr_km<KM>(); \
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rys_jk_kernel<KM>, 128, smem_of(rc, 4))
-  RYS_KM_DISPATCH(rc, RYS_O)
+    RYS_KM_DISPATCH(rc, RYS_O)
 #undef RYS_O
-  return n;
+    return n;
+  }();
+  return occ;
 }
 
 template <int CLS>

@@ -49,10 +49,13 @@ void jk_thread_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc
 }
 template <int CLS>
 int jk_thread_occ() {
-  int n = 0;
-  if constexpr (thread_class(CLS))
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<RysTOf<CLS>, double>, 128, 0);
-  return n;
+  static const int occ = [] {  // asked once per process
+    int n = 0;
+    if constexpr (thread_class(CLS))
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<RysTOf<CLS>, double>, 128, 0);
+    return n;
+  }();
+  return occ;
 }
 
 template <size_t... I>
