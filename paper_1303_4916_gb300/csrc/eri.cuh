@@ -1102,9 +1102,19 @@ inline int coop_occupancy() {
   return n;
 }
 
-// ------------------------------------------------------------- ERI tensor kernel
-// Same work decomposition; every element of the block is written to all
-// eight index permutations of the dense nbf^4 tensor G (small bases).
+// ------------------------------------------------------------- ERI tensor kernels
+// The class kernels write each quartet's block once, at (i j | k l) with i,
+// j, k, l in the order of its shell pairs (bra pair first); mirror_tensor
+// (basis.cu) then copies it to the other index permutations.  An item that
+// is split along its primitive loop adds its part into the zeroed tensor.
+// Writing all eight images from here, as it was done before, cost up to
+// eight scattered 8-byte stores per integral and forbade the split, so that
+// a quartet of two 36-primitive pairs ran on one thread.
+__device__ __forceinline__ void store_eri(double* __restrict__ G, size_t idx, double v, bool add) {
+  if (add) atomicAdd(G + idx, v);
+  else G[idx] = v;
+}
+
 template <class C>
 __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
                                                         double* __restrict__ G, int nbf) {
@@ -1122,18 +1132,17 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
     }
     const int bi = lo;
     const int bp = __ldg(w.bra + bi);
-    // the tensor is written, not accumulated: part 0 of a split item takes
-    // the whole primitive loop and the other parts do nothing
     const int nsp = w.nsplit ? __ldg(w.nsplit + bi) : 1;
     const int rr = t - __ldg(w.ioff + bi);
-    if (rr % nsp != 0) continue;
-    const int kidx = __ldg(w.kbeg + bi) + w.chunk * (rr / nsp) + lane;
-    if (lane >= w.chunk || kidx >= __ldg(w.kend + bi)) continue;
+    const int kblk = rr / nsp, part = rr - kblk * nsp;
+    const int kidx = __ldg(w.kbeg + bi) + 32 * kblk + lane;
+    if (kidx >= __ldg(w.kend + bi)) continue;
     const int kp = __ldg(w.ket + kidx);
     const PairInfo bra = ps.info[bp];
     const PairInfo ket = ps.info[kp];
+    const int ib0 = part * bra.nprim / nsp, ib1 = (part + 1) * bra.nprim / nsp;
     double acc[C::NE * C::NF];
-    contracted_vrr<C, double>(ps, kc, bra.prim0, bra.nprim, ket.prim0, ket.nprim, acc);
+    contracted_vrr<C, double>(ps, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0, ket.nprim, acc);
     double I[NA * NB * NC * ND];
     C::template hrr<double>(acc, I, bra.AB, ket.AB);
     const size_t n = (size_t)nbf;
@@ -1148,16 +1157,63 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
             const double v = I[((a * NB + b) * NC + c) * ND + d] * comp_scale(C::LA, a) * comp_scale(C::LB, b) *
                              comp_scale(C::LC, c) * comp_scale(C::LD, d);
             const size_t i = bra.bfA + a, j = bra.bfB + b, k = ket.bfA + c, l = ket.bfB + d;
-            G[((i * n + j) * n + k) * n + l] = v;
-            G[((j * n + i) * n + k) * n + l] = v;
-            G[((i * n + j) * n + l) * n + k] = v;
-            G[((j * n + i) * n + l) * n + k] = v;
-            G[((k * n + l) * n + i) * n + j] = v;
-            G[((l * n + k) * n + i) * n + j] = v;
-            G[((k * n + l) * n + j) * n + i] = v;
-            G[((l * n + k) * n + j) * n + i] = v;
+            store_eri(G, ((i * n + j) * n + k) * n + l, v, nsp > 1);
           }
   }
+}
+
+// Classes with L >= 5: one warp per quartet (part), the block from
+// coop_block.  What bounds it is what bounds the J/K kernel of the class
+// (FP64 issue).  A thread per quartet, the form before, kept the whole
+// [e0|f0] set of such a class in one thread and spilled it.
+template <class C>
+__global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
+                                                             double* __restrict__ G, int nbf, const int g) {
+  using S = CoopSizes<C>;
+  constexpr int NB = C::NB, ND = C::ND, NF = C::NF, NAB = S::NAB, NCD = S::NCD;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* const s = reinterpret_cast<double*>(smem_raw) + (threadIdx.x >> 5) * S::ws(g);
+  const int lane = threadIdx.x & 31;
+  for (;;) {
+    int t = 0;
+    if (lane == 0) t = atomicAdd(w.counter, 1);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (t >= w.nitems) break;
+    int lo = 0, hi = w.nbra;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (__ldg(w.ioff + mid) <= t) lo = mid; else hi = mid;
+    }
+    const int bp = __ldg(w.bra + lo);
+    const int nsp = w.nsplit ? __ldg(w.nsplit + lo) : 1;
+    const int rr = t - __ldg(w.ioff + lo);
+    const int kj = rr / nsp, part = rr - kj * nsp;
+    const int kp = __ldg(w.ket + __ldg(w.kbeg + lo) + kj);
+    const PairInfo bra = ps.info[bp];
+    const PairInfo ket = ps.info[kp];
+    const int nq = bra.nprim * ket.nprim;
+    coop_block<C, double>(ps.prim64, kc, bra, ket, part * nq / nsp, (part + 1) * nq / nsp, s, g, lane);
+    __syncwarp();
+    const double* const Id = s + S::NT + NAB * NF;  // scaled by the d components
+    const size_t n = (size_t)nbf;
+    for (int o = lane; o < NAB * NCD; o += 32) {
+      const int ab = o / NCD, cd = o - ab * NCD;
+      const size_t i = bra.bfA + ab / NB, j = bra.bfB + ab % NB, k = ket.bfA + cd / ND, l = ket.bfB + cd % ND;
+      store_eri(G, ((i * n + j) * n + k) * n + l, Id[o], nsp > 1);
+    }
+    __syncwarp();
+  }
+}
+
+template <class C>
+inline void store_coop_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, double* G, int nbf, int grid,
+                              cudaStream_t s) {
+  const int g = coop_group<C>();
+  const size_t sm = coop_smem_bytes<C, double>(g);
+  static const cudaError_t attr =  // set once per process
+      cudaFuncSetAttribute(eri_store_coop_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  (void)attr;
+  eri_store_coop_kernel<C><<<grid, 128, sm, s>>>(w, ps, kc, G, nbf, g);
 }
 
 // ------------------------------------------------------------- Schwarz kernel
@@ -1200,7 +1256,7 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
       hfk::eri_jk_kernel<hfgen::CLS, R><<<grid, threads, 0, s>>>(w, ps, kc, one, mols);                  \
   }                                                                                                      \
   template <typename R>                                                                                  \
-  static int occR_##CLS() {                                                                              \
+  static int occR_query_##CLS() {                                                                        \
     int n = 0;                                                                                           \
     if constexpr (hfgen::CLS::COOP)                                                                      \
       n = hfk::coop_occupancy<hfgen::CLS, R>();                                                          \
@@ -1230,7 +1286,7 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
     else                                                                                                 \
       launch_jkR_##CLS<double>(w, ps, kc, one, mols, grid, threads, s);                                  \
   }                                                                                                      \
-  static int occ_jkdf_##CLS() {                                                                          \
+  static int occ_jkdf_query_##CLS() {                                                                    \
     int n = 0;                                                                                           \
     if constexpr (hfgen::CLS::COOP)                                                                      \
       n = hfk::coop_occupancy<hfgen::CLS, df64>();                                                       \

@@ -163,6 +163,9 @@ struct hf_basis {
   // two 64-bit words per element
   DevArray<unsigned long long> detq;
 
+  // tensor path (lazily): shell of each function, rank of each oriented shell pair
+  DevArray<int> bfshell, pairkey;
+
   // one-electron data (lazily)
   DevArray<double> S, T, V;
   bool have_one = false;

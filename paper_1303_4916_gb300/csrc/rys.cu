@@ -711,9 +711,9 @@ __global__ void __launch_bounds__(128) rys_jk_kernel(const JKWork w, const PairS
   }
 }
 
-// Dense tensor: every element of each quartet's block to its eight index
-// permutations (small bases).  An s/p/d item split along its primitive
-// loop is taken whole by part 0.
+// Dense tensor: each quartet's block at the index order of its pairs (added
+// where the item covers a part of the primitive loop; mirror_tensor in
+// basis.cu copies it to the other permutations).
 template <int KM>
 __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
                                                         double* __restrict__ G, int nbf, const RysClass rc) {
@@ -728,35 +728,27 @@ __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const Pa
     if (t >= w.nitems) break;
     ItemRange it;
     rys_item(w, t, &it);
-    // the tensor is written, not accumulated: the first primitive range of
-    // each chunk takes the whole primitive loop, the other ranges do nothing
-    if (w.nchunk > 0 ? it.part >= w.nchunk : it.part != 0) continue;
     const int bp = __ldg(w.bra + it.bi);
     const PairInfo bra = ps.info[bp];
+    const bool add = it.nsp > (w.nchunk > 0 ? w.nchunk : 1);
     for (int kidx = it.k0; kidx < it.k1; ++kidx) {
       const int kp = __ldg(w.ket + kidx);
       const PairInfo ket = ps.info[kp];
-      const int c_lo = w.nchunk > 0 ? it.part : 0, c_hi = w.nchunk > 0 ? it.part + 1 : rc.nchunks;
+      int q_lo, q_hi, c_lo, c_hi;
+      rys_part(rc, w, bra, ket, it.part, it.nsp, &q_lo, &q_hi, &c_lo, &c_hi);
+      if (q_hi <= q_lo) continue;
       rys_setup(rc, bra.AB, ket.AB, s, lane);
       for (int ch = c_lo; ch < c_hi; ++ch) {
         const int r0 = ch * rc.rpc, r1 = min(r0 + rc.rpc, rc.na * NB);
-        rys_rows<KM>(rc, ps.prim64, kc.rys, bra, ket, 0, bra.nprim * ket.nprim, r0, r1, s, lane);
+        rys_rows<KM>(rc, ps.prim64, kc.rys, bra, ket, q_lo, q_hi, r0, r1, s, lane);
         const double* I = s + rc.oBlk;
         const size_t n = (size_t)nbf;
         for (int e = lane; e < (r1 - r0) * NCD; e += 32) {
           const int rl = e / NCD, cd = e - rl * NCD;
           const int row = r0 + rl, a = row / NB, b = row - a * NB;
           const int c = cd / ND, d = cd - c * ND;
-          const double v = I[e];
           const size_t i = bra.bfA + a, j = bra.bfB + b, k = ket.bfA + c, l = ket.bfB + d;
-          G[((i * n + j) * n + k) * n + l] = v;
-          G[((j * n + i) * n + k) * n + l] = v;
-          G[((i * n + j) * n + l) * n + k] = v;
-          G[((j * n + i) * n + l) * n + k] = v;
-          G[((k * n + l) * n + i) * n + j] = v;
-          G[((l * n + k) * n + i) * n + j] = v;
-          G[((k * n + l) * n + j) * n + i] = v;
-          G[((l * n + k) * n + j) * n + i] = v;
+          hfk::store_eri(G, ((i * n + j) * n + k) * n + l, I[e], add);
         }
         __syncwarp();
       }
