@@ -9,7 +9,7 @@
 //         + sum over unique quartets Gamma d(ab|cd)/dR + dE_nuc/dR,
 // the W term coming from the orthonormality of the orbitals.  The two-
 // electron part runs on the Rys derivative kernel of every class
-// (rys.cu); the one-electron part here, one thread per ordered pair (i, j)
+// (rys.cu); the one-electron part here, one warp per ordered pair (i, j)
 // of basis functions, takes the derivatives with respect to the centre A
 // of function i:
 //   d phi_a / dA_x = 2 alpha phi_(a + 1_x) - a_x phi_(a - 1_x)
@@ -17,7 +17,7 @@
 // Rys-quadrature nuclear attraction (a (i|1/r_C|j) with n = (la+lb+1)/2 + 1
 // roots).  D, W, H and S are symmetric, so over all ordered pairs the
 // derivatives with respect to the ket centre add up to those with respect
-// to the bra centre: each thread adds twice its bra-centre term,
+// to the bra centre: each pair adds twice its bra-centre term,
 //   4 D_ij dH_ij/dA - 4 W_ij dS_ij/dA  to the atom of i,
 // and the operator's own centre C (the Hellmann-Feynman term), whose
 // derivative of (i|1/r_C|j) is -(d/dA + d/dB) by translational invariance,
@@ -50,23 +50,27 @@ __device__ double comp_scale_g(int l, int c) {
   return sqrt(df(l) / (df(p[0]) * df(p[1]) * df(p[2])));
 }
 
-__device__ double binom_g(int n, int k) {
-  double r = 1.0;
-  for (int i = 1; i <= k; ++i) r = r * (n - k + i) / i;
-  return r;
+__device__ __forceinline__ double sub_add(double v, int width) {  // sum over aligned groups of `width` lanes
+  for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// thread per ordered pair (i, j): one-electron gradient terms of the
-// derivative with respect to the centre of i
-__global__ void onee_grad_kernel(int nbf, const int* __restrict__ bf_shell, const int* __restrict__ sh_l,
-                                 const int* __restrict__ sh_bf, const int* __restrict__ sh_nprim,
-                                 const int* __restrict__ sh_prim, const int* __restrict__ sh_atom,
-                                 const double* __restrict__ sh_xyz, const double* __restrict__ exps,
-                                 const double* __restrict__ coefs, int natom, const double* __restrict__ atom_xyz,
-                                 const int* __restrict__ atom_Z, const double* __restrict__ rys,
-                                 const double* __restrict__ D, const double* __restrict__ W,
-                                 double* __restrict__ grad) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+// One warp per ordered pair (i, j): the gradient terms of the derivative
+// with respect to the centre of i.  Lanes take the primitive pairs for the
+// overlap and kinetic terms; for the attraction groups of `w` lanes (w a
+// power of two, at most the primitive-pair count rounded up) each take one
+// nucleus, their lanes over its primitive pairs, so that contracted pairs
+// and single primitives both fill the warp.  FP64 issue bounds it; a thread
+// per (i, j) over all primitives and nuclei, the form before, left the GPU
+// waiting on its longest pair (45 ms at 49 functions of 5 atoms).
+__global__ void __launch_bounds__(128) onee_grad_kernel(
+    int nbf, const int* __restrict__ bf_shell, const int* __restrict__ sh_l, const int* __restrict__ sh_bf,
+    const int* __restrict__ sh_nprim, const int* __restrict__ sh_prim, const int* __restrict__ sh_atom,
+    const double* __restrict__ sh_xyz, const double* __restrict__ exps, const double* __restrict__ coefs, int natom,
+    const double* __restrict__ atom_xyz, const int* __restrict__ atom_Z, const double* __restrict__ rys,
+    const double* __restrict__ D, const double* __restrict__ W, double* __restrict__ grad) {
+  const long long t = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (t >= (long long)nbf * nbf) return;
   const int i = (int)(t / nbf), j = (int)(t % nbf);
   const double Dij = D[t], Wij = W[t];
@@ -84,104 +88,100 @@ __global__ void onee_grad_kernel(int nbf, const int* __restrict__ bf_shell, cons
     AB[x] = A[x] - B[x];
     r2 += AB[x] * AB[x];
   }
-  double gS[3] = {0, 0, 0}, gT[3] = {0, 0, 0}, gV[3] = {0, 0, 0};
-  double gVC[3 * 8];  // per nucleus, in rounds of 8
-  const int L = la + lb + 1;
-  const int nr = L / 2 + 1;
-  for (int c0 = 0; c0 < natom; c0 += 8) {
-    const int cn = min(8, natom - c0);
-    for (int k = 0; k < 3 * cn; ++k) gVC[k] = 0.0;
-    for (int ka = 0; ka < sh_nprim[sa]; ++ka)
-      for (int kb = 0; kb < sh_nprim[sb]; ++kb) {
+  const int nb = sh_nprim[sb], np = sh_nprim[sa] * nb;
+  double gA[3] = {0, 0, 0};  // 4 D (dT + dV) - 4 W dS
+  for (int k = lane; k < np; k += 32) {
+    const int ka = k / nb, kb = k - ka * nb;
+    const double a = exps[sh_prim[sa] + ka], b = exps[sh_prim[sb] + kb];
+    const double c = coefs[sh_prim[sa] + ka] * coefs[sh_prim[sb] + kb] * scale;
+    const double p = a + b, o2p = 0.5 / p, mu = a * b / p;
+    double s0[3], t0[3], sd[3], td[3];
+    for (int x = 0; x < 3; ++x) {
+      const double P = (a * A[x] + b * B[x]) / p, PA = P - A[x], PB = P - B[x];
+      double s[6][7];  // 1D overlaps, i <= la + 1, j <= lb + 2
+      s[0][0] = sqrt(3.14159265358979323846 / p) * exp(-mu * AB[x] * AB[x]);
+      for (int ii = 0; ii < pa[x] + 1; ++ii) s[ii + 1][0] = PA * s[ii][0] + (ii > 0 ? ii * o2p * s[ii - 1][0] : 0.0);
+      for (int ii = 0; ii <= pa[x] + 1; ++ii)
+        for (int jj = 0; jj < pb[x] + 2; ++jj)
+          s[ii][jj + 1] = PB * s[ii][jj] + ((ii > 0 ? ii * s[ii - 1][jj] : 0.0) + (jj > 0 ? jj * s[ii][jj - 1] : 0.0)) * o2p;
+      // kinetic factor of the ket on row ii
+      auto tk = [&](int ii) {
+        const int jj = pb[x];
+        double v = -2.0 * b * (2 * jj + 1) * s[ii][jj] + 4.0 * b * b * s[ii][jj + 2];
+        if (jj >= 2) v += jj * (jj - 1) * s[ii][jj - 2];
+        return -0.5 * v;
+      };
+      s0[x] = s[pa[x]][pb[x]];
+      t0[x] = tk(pa[x]);
+      sd[x] = 2.0 * a * s[pa[x] + 1][pb[x]] - (pa[x] > 0 ? pa[x] * s[pa[x] - 1][pb[x]] : 0.0);
+      td[x] = 2.0 * a * tk(pa[x] + 1) - (pa[x] > 0 ? pa[x] * tk(pa[x] - 1) : 0.0);
+    }
+    for (int x = 0; x < 3; ++x) {
+      const int y = x == 2 ? 0 : x + 1, z = x == 0 ? 2 : x - 1;
+      gA[x] += 4.0 * Dij * (c * (td[x] * s0[y] * s0[z] + sd[x] * (t0[y] * s0[z] + s0[y] * t0[z])));
+      gA[x] -= 4.0 * Wij * (c * sd[x] * s0[y] * s0[z]);
+    }
+  }
+  // nuclear attraction by Rys quadrature: per root, 1D factors I(i, 0) from
+  // I(i+1) = (PA - u PC) I(i) + i (1-u)/(2p) I(i-1), then I(i, j+1) =
+  // I(i+1, j) + AB I(i, j), which leaves I(pa - 1 .. pa + 1, pb)
+  const int nr = (la + lb + 1) / 2 + 1;
+  int w = 1;
+  while (w < np && w < 32) w <<= 1;
+  const int sub = lane & (w - 1);
+  for (int c0 = 0; c0 < natom; c0 += 32 / w) {
+    const int at = c0 + lane / w;
+    const bool live = at < natom && atom_Z[at < natom ? at : 0] != 0;
+    double gC[3] = {0, 0, 0};
+    if (live)
+      for (int k = sub; k < np; k += w) {
+        const int ka = k / nb, kb = k - ka * nb;
         const double a = exps[sh_prim[sa] + ka], b = exps[sh_prim[sb] + kb];
-        const double c = coefs[sh_prim[sa] + ka] * coefs[sh_prim[sb] + kb] * scale;
-        const double p = a + b, o2p = 0.5 / p, mu = a * b / p;
-        double P[3], PA[3], PB[3];
+        const double ip = 1.0 / (a + b), p = a + b, o2p = 0.5 * ip;
+        const double f = -(double)atom_Z[at] * coefs[sh_prim[sa] + ka] * coefs[sh_prim[sb] + kb] * scale *
+                         (2.0 * 3.14159265358979323846 * ip * exp(-(a * b * ip) * r2));
+        double PA[3], PC[3];
         for (int x = 0; x < 3; ++x) {
-          P[x] = (a * A[x] + b * B[x]) / p;
-          PA[x] = P[x] - A[x];
-          PB[x] = P[x] - B[x];
+          const double P = (a * A[x] + b * B[x]) * ip;
+          PA[x] = P - A[x];
+          PC[x] = P - atom_xyz[3 * at + x];
         }
-        if (c0 == 0) {
-          // 1D overlaps S[x][i][j], i <= la + 1, j <= lb + 2
-          double S1[3][6][7];
+        const double Tn = p * (PC[0] * PC[0] + PC[1] * PC[1] + PC[2] * PC[2]);
+        double dv[3] = {0, 0, 0};
+        for (int r = 0; r < nr; ++r) {
+          double u, wt;
+          rys_rule_root(rys, nr, r, Tn, &u, &wt);
+          double v0[3], vd[3];
           for (int x = 0; x < 3; ++x) {
-            double (*s)[7] = S1[x];
-            s[0][0] = sqrt(3.14159265358979323846 / p) * exp(-mu * AB[x] * AB[x]);
-            for (int ii = 0; ii < pa[x] + 1; ++ii)
-              s[ii + 1][0] = PA[x] * s[ii][0] + (ii > 0 ? ii * o2p * s[ii - 1][0] : 0.0);
-            for (int ii = 0; ii <= pa[x] + 1; ++ii)
-              for (int jj = 0; jj < pb[x] + 2; ++jj)
-                s[ii][jj + 1] = PB[x] * s[ii][jj] +
-                                ((ii > 0 ? ii * s[ii - 1][jj] : 0.0) + (jj > 0 ? jj * s[ii][jj - 1] : 0.0)) * o2p;
+            double g[11];
+            g[0] = 1.0;
+            const double c00 = PA[x] - u * PC[x], b10 = (1.0 - u) * o2p;
+            const int top = pa[x] + 1 + pb[x], lo = pa[x] > 0 ? pa[x] - 1 : 0;
+            for (int m = 0; m < top; ++m) g[m + 1] = c00 * g[m] + (m > 0 ? m * b10 * g[m - 1] : 0.0);
+            for (int m = 1; m <= pb[x]; ++m)
+              for (int e = lo; e <= top - m; ++e) g[e] = g[e + 1] + AB[x] * g[e];
+            v0[x] = g[pa[x]];
+            vd[x] = 2.0 * a * g[pa[x] + 1] - (pa[x] > 0 ? pa[x] * g[lo] : 0.0);
           }
-          // kinetic factor of the ket on row ii
-          auto tk = [&](int x, int ii) {
-            const int jj = pb[x];
-            double v = -2.0 * b * (2 * jj + 1) * S1[x][ii][jj] + 4.0 * b * b * S1[x][ii][jj + 2];
-            if (jj >= 2) v += jj * (jj - 1) * S1[x][ii][jj - 2];
-            return -0.5 * v;
-          };
-          double s0[3], t0[3], sd[3], td[3];
-          for (int x = 0; x < 3; ++x) {
-            s0[x] = S1[x][pa[x]][pb[x]];
-            t0[x] = tk(x, pa[x]);
-            sd[x] = 2.0 * a * S1[x][pa[x] + 1][pb[x]] - (pa[x] > 0 ? pa[x] * S1[x][pa[x] - 1][pb[x]] : 0.0);
-            td[x] = 2.0 * a * tk(x, pa[x] + 1) - (pa[x] > 0 ? pa[x] * tk(x, pa[x] - 1) : 0.0);
-          }
-          for (int x = 0; x < 3; ++x) {
-            const int y = (x + 1) % 3, z = (x + 2) % 3;
-            gS[x] += c * sd[x] * s0[y] * s0[z];
-            gT[x] += c * (td[x] * s0[y] * s0[z] + sd[x] * (t0[y] * s0[z] + s0[y] * t0[z]));
-          }
+          dv[0] += wt * vd[0] * v0[1] * v0[2];
+          dv[1] += wt * v0[0] * vd[1] * v0[2];
+          dv[2] += wt * v0[0] * v0[1] * vd[2];
         }
-        // nuclear attraction by Rys quadrature: per root, 1D factors
-        // I(i, j) from I(i+1) = (PA - u PC) I(i) + i (1-u)/(2p) I(i-1) and
-        // the transfer to B
-        const double pre = 2.0 * 3.14159265358979323846 / p * exp(-mu * r2);
-        for (int cc = 0; cc < cn; ++cc) {
-          const int at = c0 + cc;
-          if (atom_Z[at] == 0) continue;
-          const double* Cc = atom_xyz + 3 * at;
-          const double PC[3] = {P[0] - Cc[0], P[1] - Cc[1], P[2] - Cc[2]};
-          const double Tn = p * (PC[0] * PC[0] + PC[1] * PC[1] + PC[2] * PC[2]);
-          double dv[3] = {0, 0, 0};
-          for (int r = 0; r < nr; ++r) {
-            double u, w;
-            rys_rule_root(rys, nr, r, Tn, &u, &w);
-            double v0[3], vd[3];
-            for (int x = 0; x < 3; ++x) {
-              double g[11];
-              g[0] = 1.0;
-              const double c00 = PA[x] - u * PC[x], b10 = (1.0 - u) * o2p;
-              const int top = pa[x] + 1 + pb[x];
-              for (int k = 0; k < top; ++k) g[k + 1] = c00 * g[k] + (k > 0 ? k * b10 * g[k - 1] : 0.0);
-              auto tr = [&](int ii) {  // I(ii, pb) by the transfer to B
-                double v = 0.0;
-                for (int k = 0; k <= pb[x]; ++k) v += binom_g(pb[x], k) * pow(AB[x], pb[x] - k) * g[ii + k];
-                return v;
-              };
-              v0[x] = tr(pa[x]);
-              vd[x] = 2.0 * a * tr(pa[x] + 1) - (pa[x] > 0 ? pa[x] * tr(pa[x] - 1) : 0.0);
-            }
-            dv[0] += w * vd[0] * v0[1] * v0[2];
-            dv[1] += w * v0[0] * vd[1] * v0[2];
-            dv[2] += w * v0[0] * v0[1] * vd[2];
-          }
-          const double f = -(double)atom_Z[at] * c * pre;
-          for (int x = 0; x < 3; ++x) {
-            gV[x] += f * dv[x];
-            gVC[3 * cc + x] += f * dv[x];
-          }
-        }
+        for (int x = 0; x < 3; ++x) gC[x] += f * dv[x];
       }
+    for (int x = 0; x < 3; ++x) {
+      gA[x] += 4.0 * Dij * gC[x];
+      gC[x] = sub_add(gC[x], w);
+    }
     // the operator's centre
-    for (int cc = 0; cc < cn; ++cc)
-      for (int x = 0; x < 3; ++x)
-        if (gVC[3 * cc + x] != 0.0) atomicAdd(grad + 3 * (c0 + cc) + x, -4.0 * Dij * gVC[3 * cc + x]);
+    if (live && sub == 0)
+      for (int x = 0; x < 3; ++x) atomicAdd(grad + 3 * at + x, -4.0 * Dij * gC[x]);
   }
   const int ai = sh_atom[sa];
-  for (int x = 0; x < 3; ++x) atomicAdd(grad + 3 * ai + x, 4.0 * Dij * (gT[x] + gV[x]) - 4.0 * Wij * gS[x]);
+  for (int x = 0; x < 3; ++x) {
+    gA[x] = sub_add(gA[x], 32);
+    if (lane == 0) atomicAdd(grad + 3 * ai + x, gA[x]);
+  }
 }
 
 // rows of M = (row-major C)^T scaled by eps: Me(i, mu) = eps_i M(i, mu)
@@ -270,7 +270,7 @@ extern "C" int hf_rhf_gradient(hf_basis* b, const double* C, const double* eps, 
   UP(co, b->coefs.data(), b->nprim);
   UP(ax, at_xyz.data(), 3 * na);
 #undef UP
-  onee_grad_kernel<<<(unsigned)((nn + 127) / 128), 128, 0, st>>>(n, bfs.ptr, dl.ptr, dbf.ptr, dn.ptr, dp.ptr, dsa.ptr,
+  onee_grad_kernel<<<(unsigned)((nn + 3) / 4), 128, 0, st>>>(n, bfs.ptr, dl.ptr, dbf.ptr, dn.ptr, dp.ptr, dsa.ptr,
                                                                  sx.ptr, ex.ptr, co.ptr, na, ax.ptr, dZ.ptr, ctx->rys,
                                                                  D.ptr, W.ptr, g.ptr);
   HF_CUDA(cudaGetLastError());
