@@ -102,6 +102,49 @@ static void boys_row(long double T, long double* F, long double* et) {
   for (int m = M - 1; m >= 0; --m) F[m] = (2.0L * T * F[m + 1] + *et) / (long double)(2 * m + 1);
 }
 
+// Rows of the S_m(y) tables (hf_device.h): near rows from boys_row, far rows
+// from the large-T form F_m = sqrt(pi / T) / 2 (2m - 1)!! / (2T)^m.
+void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
+  auto split = [](long double c, float* q) {
+    q[0] = (float)c;
+    q[1] = (float)(c - (long double)q[0]);
+  };
+  long double F[BOYS_NM], et;
+  auto rows = [&](uint32_t* t, int nrow0, bool df) {  // S_m in F -> row nrow0 of every slice
+    for (int L = 0; L <= BOYSY_LMAX; ++L) {
+      uint32_t* r = t + (df ? boysydf_off(L) + (size_t)nrow0 * BOYSYDF_ROW(L) : boysy64_off(L) + (size_t)nrow0 * BOYSY64_ROW(L));
+      if (!df)
+        for (int m = 0; m <= L; ++m, r += 2) {
+          const double v = (double)F[m];
+          memcpy(r, &v, sizeof v);
+        }
+      for (int m = df ? 0 : 1; m <= L + 3; ++m, r += 2) {
+        float q[2];
+        split(F[m], q);
+        memcpy(r, q, sizeof q);
+      }
+      for (int m = L + 4; m <= L + (df ? 7 : 6); ++m, ++r) {
+        const float v = (float)F[m];
+        memcpy(r, &v, sizeof v);
+      }
+    }
+  };
+  for (int i = 0; i < BOYSY64_NNEAR; ++i) {
+    boys_row((long double)i / 64.0L, F, &et);
+    for (int m = 1; m < BOYS_NM; m += 2) F[m] = -F[m];
+    rows(t64, i, false);
+    if (i % 4 == 0) rows(tdf, i / 4, true);
+  }
+  const long double pi = 3.141592653589793238462643383279502884L;
+  for (int i = 0; i < BOYSY_NFAR; ++i) {
+    const long double T = (256 + i) / 16.0L;
+    F[0] = 0.5L * sqrtl(pi / T);
+    for (int m = 1; m < BOYS_NM; ++m) F[m] = -F[m - 1] * (2 * m - 1) / (2.0L * T);
+    rows(t64, BOYSY64_NNEAR + i, false);
+    rows(tdf, BOYSYDF_NNEAR + i, true);
+  }
+}
+
 int hf_boys_tables(hf_ctx* ctx) {
   const size_t n64 = (size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS64_ROW;
   const size_t n32 = (size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS32_ROW;
@@ -148,7 +191,16 @@ int hf_boys_tables(hf_ctx* ctx) {
       split(et, r + 14);
     }
   }
+  // S_m(y) = (-1)^m F_m(y / 2) of the Hermite kernels (layout in hf_device.h)
+  std::vector<uint32_t> ty(boysy64_off(BOYSY_LMAX + 1), 0u), tyd(boysydf_off(BOYSY_LMAX + 1), 0u);
+  hf_boysy_fill(ty.data(), tyd.data());
   void* p = nullptr;
+  HF_CHECK(hf_dev_alloc(ctx, &p, ty.size() * sizeof(uint32_t)));
+  ctx->boysy64 = (uint32_t*)p;
+  HF_CUDA(cudaMemcpyAsync(ctx->boysy64, ty.data(), ty.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
+  HF_CHECK(hf_dev_alloc(ctx, &p, tyd.size() * sizeof(uint32_t)));
+  ctx->boysydf = (uint32_t*)p;
+  HF_CUDA(cudaMemcpyAsync(ctx->boysydf, tyd.data(), tyd.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
   HF_CHECK(hf_dev_alloc(ctx, &p, ndf * sizeof(float)));
   ctx->boysdf = (float*)p;
   HF_CUDA(cudaMemcpyAsync(ctx->boysdf, tdf.data(), ndf * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
@@ -262,6 +314,8 @@ void hf_ctx_teardown(hf_ctx* c) {
   if (c->boys64) hf_dev_free(c, c->boys64, 0);
   if (c->boys32) hf_dev_free(c, c->boys32, 0);
   if (c->boysdf) hf_dev_free(c, c->boysdf, 0);
+  if (c->boysy64) hf_dev_free(c, c->boysy64, 0);
+  if (c->boysydf) hf_dev_free(c, c->boysydf, 0);
   if (c->rys) hf_dev_free(c, c->rys, 0);
   if (c->bounds) hf_dev_free(c, c->bounds, 0);
   if (c->stream) cudaStreamSynchronize(c->stream);

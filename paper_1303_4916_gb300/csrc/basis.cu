@@ -37,6 +37,7 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
                             const int* __restrict__ sh_prim, const int* __restrict__ sh_bf,
                             const double* __restrict__ exps, const double* __restrict__ coefs,
                             double* __restrict__ prim64, float* __restrict__ prim32, float* __restrict__ primdf,
+                            double* __restrict__ primh, float* __restrict__ primhdf,
                             PairInfo* __restrict__ info, double eps) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npairs) return;
@@ -88,6 +89,16 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
       const float h = __double2float_rn(r[x]);
       g[2 * x] = h;
       g[2 * x + 1] = __double2float_rn(r[x] - (double)h);
+    }
+    // record of the Hermite kernels: K'' = K 2^(1/4) (2p)^(-1/2)
+    double* rh = primh + (size_t)(base + s) * PRIMH_STRIDE;
+    float* gh = primhdf + (size_t)(base + s) * 2 * PRIMH_STRIDE;
+    const double hv[PRIMH_STRIDE] = {r[1], Px, Py, Pz, r[5], r[6], r[7], K * 1.1892071150027210667 * sqrt(r[1])};
+    for (int x = 0; x < PRIMH_STRIDE; ++x) {
+      rh[x] = hv[x];
+      const float h = __double2float_rn(hv[x]);
+      gh[2 * x] = h;
+      gh[2 * x + 1] = __double2float_rn(hv[x] - (double)h);
     }
   }
   PairInfo pi;
@@ -151,6 +162,79 @@ __global__ void finish_fixed(const unsigned long long* __restrict__ Jq, const un
     K2[ij] = s2;
     K2[ji] = s2;
   }
+}
+
+// ------------------------------------------------------------- ket units
+// The 32 lanes of a thread-per-quartet warp walk the primitives of 32 kets in
+// step, so they should be of like length; but the pairs of a class with
+// ragged contractions have up to 36 different lengths, and a bucket for each
+// left a warp with a few live lanes (a 9-atom s+p+d molecule: 1-5 kets per
+// bucket and bra, 5 to 50 times the time per primitive quartet of a uniform
+// basis).  So a ket goes into the lists as one or more units of at most
+// `cap` of its primitives, of sizes that differ by at most one (the
+// contraction is linear: every unit is digested as a quartet of its own),
+// and the units of a class are split into as few buckets of neighbouring
+// sizes as give the least lane time, sum over buckets of ceil(n / 32) times
+// the largest size.  A cap of 12 costs a digestion per 12 primitives of a
+// long ket; a basis so small that its primitive quartets do not fill the GPU
+// takes a lower one, down to 3, to have more units.
+static void build_ket_units(hf_basis* b) {
+  const int np = b->npairs;
+  long long total = 0;
+  for (int k = 0; k < np; ++k) total += b->nprim_sig_h[k];
+  const double per_warp = (double)total * total / 64.0 / (16.0 * b->ctx->num_sms);  // lane steps of a whole build
+  const int cap = (int)std::min(12.0, std::max(3.0, per_warp));
+  b->qrank.assign(np, 0);
+  b->ketu_h.clear();
+  for (int X = 0; X < HF_NPAIRCLASS; ++X) {
+    const int s0 = b->class_begin[X], s1 = b->class_begin[X + 1];
+    b->ketu_begin[X] = (int)b->ketu_h.size();
+    b->ubuckets[X].clear();
+    std::vector<int> by_q(s1 - s0);
+    std::iota(by_q.begin(), by_q.end(), s0);
+    std::stable_sort(by_q.begin(), by_q.end(), [&](int x, int y) { return b->Q_h[x] > b->Q_h[y]; });
+    long long count[13] = {};
+    for (int r = 0; r < s1 - s0; ++r) {
+      b->qrank[by_q[r]] = r;
+      const int n = b->nprim_sig_h[by_q[r]], nu = std::max(1, (n + cap - 1) / cap);
+      for (int u = 0; u < nu; ++u) ++count[(u + 1) * n / nu - u * n / nu];
+    }
+    // least lane time over the ways to cut sizes 0..12 into neighbouring
+    // buckets: best[z] for sizes below z
+    long long best[14];
+    int cut[14];
+    best[0] = 0;
+    for (int z = 1; z <= 13; ++z) {
+      best[z] = -1;
+      long long n = 0;
+      int top = 0;
+      for (int a = z - 1; a >= 0; --a) {  // last bucket: sizes a .. z - 1
+        n += count[a];
+        if (count[a] > 0 && top == 0) top = std::max(1, a);
+        const long long t = best[a] + (n + 31) / 32 * top;
+        if (best[z] < 0 || t < best[z]) {
+          best[z] = t;
+          cut[z] = a;
+        }
+      }
+    }
+    b->ubuckets[X].push_back(0);
+    for (int z = 13; z > 0; z = cut[z]) {
+      for (int r = 0; r < s1 - s0; ++r) {
+        const int n = b->nprim_sig_h[by_q[r]], nu = std::max(1, (n + cap - 1) / cap);
+        for (int u = 0; u < nu; ++u) {
+          const int k0 = u * n / nu, k1 = (u + 1) * n / nu;
+          if (k1 - k0 >= cut[z] && k1 - k0 < z) b->ketu_h.push_back(make_int2(by_q[r], k0 << 16 | (k1 - k0)));
+        }
+      }
+      const int end = (int)b->ketu_h.size() - b->ketu_begin[X];
+      if (end > b->ubuckets[X].back()) b->ubuckets[X].push_back(end);
+    }
+  }
+  // the pairs whole, in the order of the pair list: the FP32 ranges (an FP32
+  // sum cut in other places rounds differently)
+  b->ketw_begin = (int)b->ketu_h.size();
+  for (int k = 0; k < np; ++k) b->ketu_h.push_back(make_int2(b->ketlist_h[k], b->nprim_sig_h[b->ketlist_h[k]]));
 }
 
 // ------------------------------------------------------------- basis create
@@ -294,7 +378,9 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
         (rc = dbf.alloc(ctx, nshell + 1)) || (rc = dxyz.alloc(ctx, 3 * nshell)) || (rc = dexp.alloc(ctx, nprim)) ||
         (rc = dcoef.alloc(ctx, nprim)) || (rc = b->prim64.alloc(ctx, (size_t)off * PRIM64_STRIDE)) ||
         (rc = b->prim32.alloc(ctx, (size_t)off * PRIM32_STRIDE)) ||
-        (rc = b->primdf.alloc(ctx, (size_t)off * PRIMDF_STRIDE)) || (rc = b->pinfo.alloc(ctx, np)) ||
+        (rc = b->primdf.alloc(ctx, (size_t)off * PRIMDF_STRIDE)) ||
+        (rc = b->primh.alloc(ctx, (size_t)off * PRIMH_STRIDE)) ||
+        (rc = b->primhdf.alloc(ctx, (size_t)off * 2 * PRIMH_STRIDE)) || (rc = b->pinfo.alloc(ctx, np)) ||
         (rc = b->Q.alloc(ctx, np)) || (rc = b->ketlist.alloc(ctx, np)) || (rc = b->counters.alloc(ctx, 2 * HF_NCLASS)))
       break;
 #define UP(dst, src, cnt)                                                                                      \
@@ -314,7 +400,8 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
     UP(dcoef, b->coefs.data(), nprim);
 #undef UP
     pair_kernel<<<(np + 127) / 128, 128, 0, st>>>(np, dA.ptr, dB.ptr, dOff.ptr, dxyz.ptr, dl.ptr, dn.ptr, dp.ptr, dbf.ptr,
-                                                  dexp.ptr, dcoef.ptr, b->prim64.ptr, b->prim32.ptr, b->primdf.ptr,
+                                                  dexp.ptr, dcoef.ptr, b->prim64.ptr, b->prim32.ptr, b->primdf.ptr, b->primh.ptr,
+                                                  b->primhdf.ptr,
                                                   b->pinfo.ptr, kPrimEps);
     if (cudaGetLastError() != cudaSuccess) { rc = hf_fail(HF_ERR_CUDA, "pair_kernel launch"); break; }
     // Schwarz factors per pair class, using the (X|X) diagonal quartets.
@@ -362,8 +449,12 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
           b->buckets[X].push_back(k - s0);
       b->buckets[X].push_back(s1 - s0);
     }
+    build_ket_units(b);
+    if ((rc = b->ketu.alloc(ctx, b->ketu_h.size()))) break;
     if (cudaMemcpyAsync(b->ketlist.ptr, b->ketlist_h.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st) !=
-        cudaSuccess) {
+            cudaSuccess ||
+        cudaMemcpyAsync(b->ketu.ptr, b->ketu_h.data(), sizeof(int2) * b->ketu_h.size(), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess) {
       rc = hf_fail(HF_ERR_CUDA, "upload");
       break;
     }
@@ -392,7 +483,7 @@ extern "C" int hf_basis_nshell(const hf_basis* b) { return b ? b->nshell : 0; }
 
 extern "C" size_t hf_basis_device_bytes(const hf_basis* b) {
   if (!b) return 0;
-  size_t s = b->prim64.bytes() + b->prim32.bytes() + b->primdf.bytes() + b->pinfo.bytes() + b->Q.bytes() + b->ketlist.bytes() +
+  size_t s = b->prim64.bytes() + b->prim32.bytes() + b->primdf.bytes() + b->primh.bytes() + b->primhdf.bytes() + b->ketu.bytes() + b->pinfo.bytes() + b->Q.bytes() + b->ketlist.bytes() +
              b->counters.bytes() + b->hD.bytes() + b->hJ.bytes() + b->hK.bytes() + b->Dsum.bytes() + b->detq.bytes() + b->bfshell.bytes() + b->pairkey.bytes() + b->S.bytes() + b->T.bytes() +
              b->V.bytes();
   for (int c = 0; c < HF_NCLASS; ++c)
@@ -415,11 +506,12 @@ extern "C" int hf_schwarz(hf_basis* b, double* Q) {
 
 // ------------------------------------------------------------- work lists
 // For each canonical class (X|Y), X >= Y: every pair of class X is a bra;
-// its kets are taken bucket by bucket from the class-Y list.  Inside a
-// bucket (Q descending) the kept kets are the prefix with Q_i Q_k >= tau
-// (the Schwarz rule: drop iff Q_ab Q_cd < tau); when X == Y only kets at
-// list positions <= the bra's own position are taken, so each unordered
-// pair of pairs appears once.  Kets with Q_i Q_k >= fp32_bound form the
+// its kets are taken bucket by bucket from the class-Y list (pairs, or ket
+// units for the lists of 32 kets per item).  Inside a bucket (Q descending)
+// the kept kets are the prefix with Q_i Q_k >= tau (the Schwarz rule: drop
+// iff Q_ab Q_cd < tau); when X == Y only kets whose place in the class by Q
+// (in the list, for the FP32 range) is not below the bra's own are taken, a
+// prefix as well, so each unordered pair of pairs appears once.  Kets with Q_i Q_k >= fp32_bound form the
 // FP64 range of the entry, the rest its FP32 range.
 int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned flags) {
   const bool rys = (flags & HF_JK_RYS) != 0;
@@ -430,43 +522,55 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
     for (int Y = 0; Y <= X; ++Y) {
       const int cls = X * (X + 1) / 2 + Y;
       const int xb = b->class_begin[X], xe = b->class_begin[X + 1];
-      const int yb = b->class_begin[Y];
-      const std::vector<int>& bk = b->buckets[Y];
       // Rys lists (f/g classes, or every class under HF_JK_RYS): one ket
       // per item, each item split into the class's output chunks
       const bool rys_list = rys || (ctx->ops[cls].rys_native && ctx->ops[cls].chunk == 1);
       const int chunk = rys_list ? 1 : ctx->ops[cls].chunk;
       const int nchunk = rys_list ? ctx->ops[cls].rys_nchunks : 0;
       std::vector<int> bra[2], kb[2], ke[2], io[2], sp[2];
+      std::vector<int> kprim[2];  // largest primitive count of the entry's bucket
       long long nq[2] = {0, 0};
       io[0].push_back(0);
       io[1].push_back(0);
-      for (int i = xb; i < xe; ++i) {
-        const int pi = b->ketlist_h[i];
-        const double qi = b->Q_h[pi];
-        const int ipos = i - xb;  // the bra's position in the class-X list (== class-Y list when X == Y)
-        for (size_t u = 0; u + 1 < bk.size(); ++u) {
-          const int b0 = bk[u], b1 = bk[u + 1];
-          if (X == Y && b0 > ipos) break;
-          auto count_ge = [&](double thr) {  // first position in [b0, b1) with qi * Q < thr
-            int lo = b0, hi = b1;
-            while (lo < hi) {
-              const int mid = (lo + hi) / 2;
-              if (qi * b->Q_h[b->ketlist_h[yb + mid]] >= thr) lo = mid + 1; else hi = mid;
-            }
-            return lo;
-          };
-          int n = count_ge(tau);
-          if (X == Y) n = std::min(n, ipos + 1);
-          const int m = fp32_bound > 0.0 ? std::min(count_ge(fp32_bound), n) : n;
-          const int lo_[2] = {b0, m}, hi_[2] = {m, n};
-          for (int r = 0; r < 2; ++r) {
-            const int cnt = hi_[r] - lo_[r];
-            if (cnt <= 0) continue;
+      for (int r = 0; r < (fp32_bound > 0.0 ? 2 : 1); ++r) {
+        const bool units = chunk == 32 && r == 0;
+        const std::vector<int>& bk = units ? b->ubuckets[Y] : b->buckets[Y];
+        const int yb = b->class_begin[Y], ub = b->ketu_begin[Y];
+        auto pair_at = [&](int pos) { return units ? b->ketu_h[ub + pos].x : b->ketlist_h[yb + pos]; };
+        auto prims_at = [&](int pos) { return units ? b->ketu_h[ub + pos].y & 0xffff : b->nprim_sig_h[pair_at(pos)]; };
+        // positions of whole pairs in the unit list
+        const int shift = chunk == 32 && r == 1 ? b->ketw_begin + yb - ub : 0;
+        std::vector<int> bucket_prims(bk.empty() ? 0 : bk.size() - 1, 0);
+        for (size_t u = 0; u + 1 < bk.size(); ++u)
+          for (int k = bk[u]; k < bk[u + 1]; ++k) bucket_prims[u] = std::max(bucket_prims[u], prims_at(k));
+        for (int i = xb; i < xe; ++i) {
+          const int pi = b->ketlist_h[i];
+          const double qi = b->Q_h[pi];
+          for (size_t u = 0; u + 1 < bk.size(); ++u) {
+            const int b0 = bk[u], b1 = bk[u + 1];
+            auto prefix = [&](auto&& keep) {  // first position in [b0, b1) that is not kept
+              int lo = b0, hi = b1;
+              while (lo < hi) {
+                const int mid = (lo + hi) / 2;
+                if (keep(mid)) lo = mid + 1; else hi = mid;
+              }
+              return lo;
+            };
+            auto count_ge = [&](double thr) { return prefix([&](int k) { return qi * b->Q_h[pair_at(k)] >= thr; }); };
+            int n = count_ge(tau);
+            if (X == Y && r == 0) n = std::min(n, prefix([&](int k) { return b->qrank[pair_at(k)] <= b->qrank[pi]; }));
+            if (X == Y && r == 1) n = std::min(n, std::max(b0, i - xb + 1));
+            const int m = fp32_bound > 0.0 ? std::min(count_ge(fp32_bound), n) : n;
+            const int lo = r == 0 ? b0 : m, hi = r == 0 ? m : n;
+            if (hi <= lo) continue;
             bra[r].push_back(pi);
-            kb[r].push_back(lo_[r]);
-            ke[r].push_back(hi_[r]);
-            nq[r] += cnt;
+            kb[r].push_back(lo + shift);
+            ke[r].push_back(hi + shift);
+            kprim[r].push_back(bucket_prims[u]);
+            if (units)  // a quartet counts with the first of its units
+              for (int k = lo; k < hi; ++k) nq[r] += (b->ketu_h[ub + k].y >> 16) == 0;
+            else
+              nq[r] += hi - lo;
           }
         }
       }
@@ -479,19 +583,17 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
       // for the warp-cooperative ones, any primitive-quartet range for the
       // Rys kernel (whose items are further multiplied by its output
       // chunks).  Large workloads are not split.
-      const int yb_ = b->class_begin[Y];
       for (int r = 0; r < 2; ++r) {
         const size_t ne = bra[r].size();
         std::vector<long long> len(ne);
         long long work = 0;
         for (size_t e = 0; e < ne; ++e) {
           const long long nbp = b->nprim_sig_h[bra[r][e]];
-          const long long nkp = b->nprim_sig_h[b->ketlist_h[yb_ + kb[r][e]]];  // uniform inside a bucket
-          len[e] = nbp * nkp;  // primitive quartets per lane (per warp for the cooperative kernels)
+          len[e] = nbp * kprim[r][e];  // primitive quartets per lane (per warp for the cooperative kernels)
           work += len[e] * ((ke[r][e] - kb[r][e] + chunk - 1) / chunk) * std::max(1, nchunk);
         }
         const long long warps = 16LL * ctx->num_sms;
-        const long long floor_len = rys_list ? 16 : chunk == 1 ? 64 : 16;
+        const long long floor_len = rys_list ? 16 : chunk == 1 ? 64 : r == 0 ? 6 : 16;
         const long long target = std::max(floor_len, work / std::max(1LL, warps));
         sp[r].resize(ne);
         for (size_t e = 0; e < ne; ++e) {
@@ -525,7 +627,8 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
           HF_CUDA(cudaMemcpyAsync(w.nsplit.ptr, sp[r].data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
         }
         w.w.bra = w.bra.ptr;
-        w.w.ket = b->ketlist.ptr + yb;
+        w.w.ket = b->ketlist.ptr + b->class_begin[Y];
+        w.w.ketu = b->ketu.ptr + b->ketu_begin[Y];
         w.w.kbeg = w.kbeg.ptr;
         w.w.kend = w.kend.ptr;
         w.w.ioff = w.ioff.ptr;
@@ -695,9 +798,10 @@ extern "C" int hf_class_stats_get(hf_basis* b, const hf_jk_opts* opts, hf_class_
   std::lock_guard<std::mutex> lk(b->ctx->mu);
   cudaSetDevice(b->ctx->device);
   HF_CHECK(hf_basis_prepare_work(b, o.schwarz_tau, o.fp32_bound, o.flags));
-  // prefix sums of significant primitive-pair counts along each class's ket list
-  std::vector<long long> pre(b->npairs + 1, 0);
+  // prefix sums of significant primitive-pair counts along each class's ket lists
+  std::vector<long long> pre(b->npairs + 1, 0), preu(b->ketu_h.size() + 1, 0);
   for (int k = 0; k < b->npairs; ++k) pre[k + 1] = pre[k] + b->nprim_sig_h[b->ketlist_h[k]];
+  for (size_t k = 0; k < b->ketu_h.size(); ++k) preu[k + 1] = preu[k] + (b->ketu_h[k].y & 0xffff);
   for (int X = 0; X < HF_NPAIRCLASS; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       const int c = X * (X + 1) / 2 + Y;
@@ -713,15 +817,17 @@ extern "C" int hf_class_stats_get(hf_basis* b, const hf_jk_opts* opts, hf_class_
       const int nblk = ((st.la + 1) * (st.la + 2) / 2) * ((st.lb + 1) * (st.lb + 2) / 2) *
                        ((st.lc + 1) * (st.lc + 2) / 2) * ((st.ld + 1) * (st.ld + 2) / 2);
       st.digest_flops = 6 * 2 * nblk;
-      const int yb = b->class_begin[Y];
       for (int r = 0; r < 2; ++r) {
         ClassWork& w = r == 0 ? b->work64[c] : b->work32[c];
+        const bool units = w.w.chunk == 32;
+        const int yb = units ? b->ketu_begin[Y] : b->class_begin[Y];
+        const std::vector<long long>& ps = units ? preu : pre;
         const std::vector<int>& bra = w.bra_h;
         const std::vector<int>& kb = w.kbeg_h;
         const std::vector<int>& ke = w.kend_h;
         long long pq = 0;
         for (int i = 0; i < w.w.nbra; ++i)
-          pq += (long long)b->nprim_sig_h[bra[i]] * (pre[yb + ke[i]] - pre[yb + kb[i]]);
+          pq += (long long)b->nprim_sig_h[bra[i]] * (ps[yb + ke[i]] - ps[yb + kb[i]]);
         if (r == 0) { st.quartets_fp64 = w.nquartets; st.prim_quartets_fp64 = pq; }
         else { st.quartets_fp32 = w.nquartets; st.prim_quartets_fp32 = pq; }
       }
@@ -877,10 +983,9 @@ int hf_eri_tensor_device(hf_basis* b, double* G) {
   const size_t nn = (size_t)n * n;
   if (b->pairkey.n == 0) {
     std::vector<int> key((size_t)ns * ns, 0), bfs(n);
-    for (int k = 0; k < b->npairs; ++k) {  // rank: position in the ket lists, ascending by class
-      const int p = b->ketlist_h[k];
-      key[(size_t)b->pair_A[p] * ns + b->pair_B[p]] = k + 1;
-    }
+    for (int X = 0; X < HF_NPAIRCLASS; ++X)  // rank as in the work lists: by class, then by Q
+      for (int p = b->class_begin[X]; p < b->class_begin[X + 1]; ++p)
+        key[(size_t)b->pair_A[p] * ns + b->pair_B[p]] = b->class_begin[X] + b->qrank[p] + 1;
     for (int s = 0; s < ns; ++s)
       for (int k = b->sh_bf[s]; k < b->sh_bf[s + 1]; ++k) bfs[k] = s;
     HF_CHECK(b->bfshell.alloc(ctx, n));

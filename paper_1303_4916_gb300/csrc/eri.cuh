@@ -26,6 +26,7 @@
 
 #include "df64.cuh"
 #include "eri_classes.cuh"
+#include "herm.cuh"
 #include "hf_device.h"
 #include "rys.cuh"
 
@@ -308,40 +309,6 @@ __device__ __forceinline__ void load_prim_df(const float* __restrict__ base, int
   q.K = df64(e.x, e.y);
 }
 
-template <class C>
-__device__ __forceinline__ void contracted_vrr_df(const PairSet& ps, const KernelCommon& kc, int b0, int nb, int k0,
-                                                  int nk, df64* acc) {
-#pragma unroll
-  for (int x = 0; x < C::NE * C::NF; ++x) acc[x] = df64(0.0f, 0.0f);
-  for (int ik = 0; ik < nk; ++ik) {
-    Prim<df64> c;
-    load_prim_df(ps.primdf, k0 + ik, c);
-    for (int ib = 0; ib < nb; ++ib) {
-      Prim<df64> a;
-      load_prim_df(ps.primdf, b0 + ib, a);
-      const df64 pq = a.p + c.p;
-      const df64 rs = rsqrt(pq);
-      const df64 inv = rs * rs;
-      const df64 rp = c.p * inv;  // rho / zeta
-      const df64 rq = a.p * inv;  // rho / eta
-      df64 PQ[3], WP[3], WQ[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        PQ[i] = a.P[i] - c.P[i];
-        WP[i] = -(rp * PQ[i]);
-        WQ[i] = rq * PQ[i];
-      }
-      const df64 T = a.p * rp * (PQ[0] * PQ[0] + PQ[1] * PQ[1] + PQ[2] * PQ[2]);
-      df64 B[C::L + 1];
-      boys_df<C::L>(T, kc.boysdf, B);
-      const df64 pref = a.K * c.K * rs;
-#pragma unroll
-      for (int m = 0; m <= C::L; ++m) B[m] = B[m] * pref;
-      C::template vrr<df64>(acc, B, a.PA, WP, c.PA, WQ, a.o2p, c.o2p, df_scale2(inv, 0.5f), rp, rq);
-    }
-  }
-}
-
 // Cartesian component scale relative to the axial component,
 // sqrt((2l-1)!! / ((2x-1)!! (2y-1)!! (2z-1)!!)), components ordered x power
 // descending then y: d xy, xz, yz carry sqrt(3); f xyz sqrt(15), the
@@ -383,11 +350,12 @@ __host__ __device__ constexpr double binom_c(int n, int k) {
 // (the recurrences of rys.cu with every size known at compile time, so the
 // tables stay in registers): over the bra primitive pairs [ib0, ib1) and
 // all ket primitives, per root the three G(n, m) tables, the transfer to
-// B and D, and the Ix Iy Iz products, into I[(a NB + b) NC ND + c ND + d]
+// B and D, and the Ix Iy Iz products (ket records [k0, k0 + nk)), into I[(a NB + b) NC ND + c ND + d]
 // (component scales not applied).  Inactive lanes return zeros.
 template <class C>
 __device__ __forceinline__ void rys_thread_block(const PairSet& P, const KernelCommon& kc, const PairInfo& bra,
-                                                 const PairInfo& ket, int ib0, int ib1, bool active, double* I) {
+                                                 const PairInfo& ket, int ib0, int ib1, int k0, int nk, bool active,
+                                                 double* I) {
   constexpr int LA = C::LA, LB = C::LB, LC = C::LC, LD = C::LD;
   constexpr int NA = C::NA, NB = C::NB, NC = C::NC, ND = C::ND;
   constexpr int NMAX = LA + LB, MMAX = LC + LD, NR = (LA + LB + LC + LD) / 2 + 1;
@@ -405,7 +373,6 @@ __device__ __forceinline__ void rys_thread_block(const PairSet& P, const KernelC
 #pragma unroll
     for (int k = 1; k <= LD; ++k) CDp[d][k] = CDp[d][k - 1] * ket.AB[d];
   }
-  const int nk = ket.nprim;
   for (int ib = ib0; ib < ib1; ++ib) {
     const double* rb = P.prim64 + (size_t)(bra.prim0 + ib) * PRIM64_STRIDE;
     const double p = __ldg(rb), hp = __ldg(rb + 1);
@@ -413,7 +380,7 @@ __device__ __forceinline__ void rys_thread_block(const PairSet& P, const KernelC
     const double PA[3] = {__ldg(rb + 5), __ldg(rb + 6), __ldg(rb + 7)};
     const double Kab = __ldg(rb + 8);
     for (int ik = 0; ik < nk; ++ik) {
-      const double* rk = P.prim64 + (size_t)(ket.prim0 + ik) * PRIM64_STRIDE;
+      const double* rk = P.prim64 + (size_t)(k0 + ik) * PRIM64_STRIDE;
       const double q = __ldg(rk), hq = __ldg(rk + 1);
       const double PQ[3] = {Pp[0] - __ldg(rk + 2), Pp[1] - __ldg(rk + 3), Pp[2] - __ldg(rk + 4)};
       const double QC[3] = {__ldg(rk + 5), __ldg(rk + 6), __ldg(rk + 7)};
@@ -533,7 +500,7 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
     const MolJK* mjp = mols ? mols + __ldg(w.mol + bi) : nullptr;
     if (mjp && !mjp->active) continue;  // warp-uniform: the entry is shared by the warp
     const PairSet P = mjp ? mjp->ps : ps;
-    const int* ketb = mjp ? mjp->ketlist + mjp->ket_off[pair_class(C::LC, C::LD)] : w.ket;
+    const int2* ketb = mjp ? mjp->ketu + mjp->ketu_off[pair_class(C::LC, C::LD)] : w.ketu;
     const int bp = __ldg(w.bra + bi);
     const int nsp = w.nsplit ? __ldg(w.nsplit + bi) : 1;
     const int rr = t - __ldg(w.ioff + bi);
@@ -542,13 +509,16 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
     if (!HF_BCHECK(kc, bp >= 0 && bp < P.npairs, HF_BC_PAIR, bp)) continue;
     bool active = kidx < __ldg(w.kend + bi);
     if (active && !HF_BCHECK(kc, kidx >= 0, HF_BC_ITEM, kidx)) active = false;
-    int kp = active ? __ldg(ketb + kidx) : bp;
+    int2 unit = active ? __ldg(ketb + kidx) : make_int2(bp, 0);
+    int kp = unit.x;
     if (active && !HF_BCHECK(kc, kp >= 0 && kp < P.npairs, HF_BC_PAIR, kp)) {
       active = false;
       kp = bp;
     }
     const PairInfo bra = P.info[bp];
     const PairInfo ket = P.info[kp];
+    const int k0 = ket.prim0 + (unit.y >> 16);  // this lane's ket primitives
+    int nk = unit.y & 0xffff;
     {
       const int nbf_ = mjp ? mjp->nbf : one.nbf;
       (void)nbf_;
@@ -558,9 +528,11 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
       if (!bra_ok) continue;  // warp-uniform
       if (active && !(HF_BCHECK(kc, ket.prim0 >= 0 && ket.prim0 + ket.nprim <= P.nprimpairs, HF_BC_PRIM,
                                 ket.prim0) &&
+                      HF_BCHECK(kc, (unit.y >> 16) + nk <= ket.nprim, HF_BC_PRIM, unit.y) &&
                       HF_BCHECK(kc, ket.bfA + NC <= nbf_ && ket.bfB + ND <= nbf_, HF_BC_MAT, ket.bfA)))
         active = false;
     }
+    if (!active) nk = 0;
     // this part's bra primitive pairs (all of them unless the item is split;
     // the contraction is linear, so the parts' digested blocks add up)
     const int ib0 = part * bra.nprim / nsp, ib1 = (part + 1) * bra.nprim / nsp;
@@ -568,13 +540,13 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
     R I[NA * NB * NC * ND];
     if constexpr (IsRys<C>::value) {
       static_assert(std::is_same<R, double>::value, "Rys thread classes run in FP64");
-      rys_thread_block<C>(P, kc, bra, ket, ib0, ib1, active, I);
+      rys_thread_block<C>(P, kc, bra, ket, ib0, ib1, k0, nk, active, I);
     } else {
       R acc[C::NE * C::NF];
-      if constexpr (std::is_same<R, df64>::value)
-        contracted_vrr_df<C>(P, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0, active ? ket.nprim : 0, acc);
+      if constexpr (std::is_same<R, float>::value)
+        contracted_vrr<C, R>(P, kc, bra.prim0 + ib0, ib1 - ib0, k0, nk, acc);
       else
-        contracted_vrr<C, R>(P, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0, active ? ket.nprim : 0, acc);
+        contracted<C, R>(P, kc, bra.prim0 + ib0, ib1 - ib0, k0, nk, acc);
       R AB[3] = {(R)bra.AB[0], (R)bra.AB[1], (R)bra.AB[2]};
       R CD[3] = {(R)ket.AB[0], (R)ket.AB[1], (R)ket.AB[2]};
       C::template hrr<R>(acc, I, AB, CD);
@@ -1137,12 +1109,13 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
     const int kblk = rr / nsp, part = rr - kblk * nsp;
     const int kidx = __ldg(w.kbeg + bi) + 32 * kblk + lane;
     if (kidx >= __ldg(w.kend + bi)) continue;
-    const int kp = __ldg(w.ket + kidx);
+    const int2 unit = __ldg(w.ketu + kidx);
     const PairInfo bra = ps.info[bp];
-    const PairInfo ket = ps.info[kp];
+    const PairInfo ket = ps.info[unit.x];
+    const bool add = nsp > 1 || (unit.y & 0xffff) < ket.nprim;
     const int ib0 = part * bra.nprim / nsp, ib1 = (part + 1) * bra.nprim / nsp;
     double acc[C::NE * C::NF];
-    contracted_vrr<C, double>(ps, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0, ket.nprim, acc);
+    contracted<C, double>(ps, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0 + (unit.y >> 16), unit.y & 0xffff, acc);
     double I[NA * NB * NC * ND];
     C::template hrr<double>(acc, I, bra.AB, ket.AB);
     const size_t n = (size_t)nbf;
@@ -1157,7 +1130,7 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
             const double v = I[((a * NB + b) * NC + c) * ND + d] * comp_scale(C::LA, a) * comp_scale(C::LB, b) *
                              comp_scale(C::LC, c) * comp_scale(C::LD, d);
             const size_t i = bra.bfA + a, j = bra.bfB + b, k = ket.bfA + c, l = ket.bfB + d;
-            store_eri(G, ((i * n + j) * n + k) * n + l, v, nsp > 1);
+            store_eri(G, ((i * n + j) * n + k) * n + l, v, add);
           }
   }
 }

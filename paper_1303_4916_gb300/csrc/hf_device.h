@@ -25,6 +25,24 @@
 #define BOYSDF_INV_H 16.0f
 #define BOYSDF_NGRID 962
 #define BOYSDF_ROW 16
+// Tables of S_m(y) = (-1)^m F_m(y / 2) for the Hermite kernels (herm.cuh), one
+// slice per L, rows of 32-bit words padded to 32 bytes.  The near rows are at
+// y_i = i / 32 (FP64) or i / 8 (df64), y < 120; after them the far rows, of the
+// large-argument form, at y_i = i / 8, i = 256 .. 1024.  A FP64 row holds
+// S_0..S_L as doubles, S_1..S_{L+3} as (hi, lo) float pairs and S_{L+4..L+6}
+// as floats; a df64 row S_0..S_{L+3} as pairs and S_{L+4..L+7} as floats.
+#define BOYSY_LMAX 4
+#define BOYSY64_NNEAR 3841
+#define BOYSYDF_NNEAR 961
+#define BOYSY_NFAR 769
+#define BOYSY64_ROW(L) ((4 * (L) + 11 + 7) / 8 * 8)
+#define BOYSYDF_ROW(L) ((2 * (L) + 12 + 7) / 8 * 8)
+__host__ __device__ constexpr size_t boysy64_off(int L) {
+  return L == 0 ? 0 : boysy64_off(L - 1) + (size_t)(BOYSY64_NNEAR + BOYSY_NFAR) * BOYSY64_ROW(L - 1);
+}
+__host__ __device__ constexpr size_t boysydf_off(int L) {
+  return L == 0 ? 0 : boysydf_off(L - 1) + (size_t)(BOYSYDF_NNEAR + BOYSY_NFAR) * BOYSYDF_ROW(L - 1);
+}
 // thread-per-quartet classes with L = la+lb+lc+ld up to this have a df64
 // variant; the warp-cooperative classes (L >= 5) take df64 through the
 // generic cooperative kernel
@@ -40,6 +58,10 @@
 #define PRIM64_STRIDE 10
 #define PRIM32_STRIDE 12
 #define PRIMDF_STRIDE 20
+// Record of the Hermite kernels: 1/(2p), P[3], PA[3], K'' = K 2^(1/4) (2p)^(-1/2)
+// (64 bytes; as (hi, lo) float pairs in df64).  With s = 1/(2p) + 1/(2q) the
+// prefactor K_ab K_cd / sqrt(p+q) is K''_ab K''_cd / sqrt(s).
+#define PRIMH_STRIDE 8
 
 // Shell pair (A, B) with l_A >= l_B: first basis functions of A and B,
 // offset and count of its significant primitive pairs (sorted by
@@ -57,6 +79,8 @@ struct PairSet {
   const float* primdf;
   int npairs;      // shell pairs (records of info)
   int nprimpairs;  // primitive-pair records
+  const double* primh;   // Hermite-kernel records, same order as prim64
+  const float* primhdf;
 };
 
 #define HF_NPAIRCLASS 15  // (la, lb), la >= lb, l <= 4
@@ -77,6 +101,8 @@ struct MolJK {
   PairSet ps;
   const int* ketlist;
   int ket_off[HF_NPAIRCLASS];
+  const int2* ketu;               // ket units (32-ket lists), and where each pair class starts
+  int ketu_off[HF_NPAIRCLASS];
   const double* Dj;
   const double* D2;
   double* K2;
@@ -91,6 +117,8 @@ struct KernelCommon {
   int det;        // J/K outputs are fixed-point integer accumulators (deterministic order)
   int* status;    // bounds-checked builds: first failed check (code, then the index), else unused
   const double* rys;  // Rys roots and weights table (rys.cuh layout)
+  const unsigned* boysy64;  // S_m(y) tables of the Hermite kernels
+  const unsigned* boysydf;
 };
 
 // Bounds-checked build (-DHF_BOUNDS_CHECK, small cases in place of a memory
@@ -113,11 +141,15 @@ struct KernelCommon {
 #define HF_BC_BOYS 5   // Boys table row
 
 // Work list of one (class, precision) launch.  Entry e pairs bra pair
-// bra[e] with the kets ket[kbeg[e] .. kend[e]) of the ket class list
-// (significant-primitive-count buckets, Schwarz-descending inside each).
+// bra[e] with the kets kbeg[e] .. kend[e] of the ket class's list: one pair
+// per position (ket) for lists of one ket per item, one ket unit per
+// position (ketu) for lists of 32.  A ket unit is a range of a pair's
+// significant primitive pairs: .x the pair, .y = first << 16 | count.
+// Lists are in buckets of like primitive count, Schwarz-descending inside.
 struct JKWork {
   const int* bra;   // [nbra] bra pair ids
-  const int* ket;   // ket list of the ket class (single-molecule launches)
+  const int* ket;   // ket pairs of the ket class (single-molecule launches)
+  const int2* ketu; // ket units of the ket class (single-molecule launches)
   const int* kbeg;  // [nbra] first ket index of each entry
   const int* kend;  // [nbra] one past the last ket index
   const int* ioff;  // [nbra+1] first work item of each entry (32 kets per item, times nsplit)

@@ -41,6 +41,8 @@ struct hf_ctx {
   double* boys64 = nullptr;
   float* boys32 = nullptr;
   float* boysdf = nullptr;
+  uint32_t* boysy64 = nullptr;  // S_m(y) of the Hermite kernels (hf_device.h)
+  uint32_t* boysydf = nullptr;
   double* rys = nullptr;    // Rys roots and weights table (rys.cuh)
   EriClassOps ops[HF_NCLASS] = {};
   static constexpr int kSide = 8;
@@ -140,6 +142,8 @@ struct hf_basis {
   DevArray<double> prim64;
   DevArray<float> prim32;
   DevArray<float> primdf;
+  DevArray<double> primh;             // records of the Hermite kernels, FP64 and (hi, lo) floats
+  DevArray<float> primhdf;
   DevArray<PairInfo> pinfo;
   DevArray<double> Q;                 // per pair
   std::vector<double> Q_h;
@@ -147,6 +151,13 @@ struct hf_basis {
   DevArray<int> ketlist;              // per pair class: pair ids, primitive-count buckets, Q descending
   std::vector<int> ketlist_h;
   std::vector<int> buckets[HF_NPAIRCLASS];  // bucket boundaries (positions in the class list)
+  std::vector<int> qrank;             // per pair: place in its class by Q descending (ties by id)
+  // ket units of the 32-ket lists (JKWork::ketu), per pair class in buckets of like size, Q descending
+  DevArray<int2> ketu;
+  std::vector<int2> ketu_h;
+  int ketu_begin[HF_NPAIRCLASS] = {};
+  int ketw_begin = 0;                 // then the pairs whole, in ketlist order
+  std::vector<int> ubuckets[HF_NPAIRCLASS];
 
   // work lists for (tau, fp32_bound)
   bool have_work = false;
@@ -177,7 +188,8 @@ struct hf_basis {
 int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned flags);
 
 inline PairSet hf_pairset(const hf_basis* b) {
-  return PairSet{b->prim64.ptr, b->prim32.ptr, b->pinfo.ptr, b->primdf.ptr, b->npairs, b->nprimpairs};
+  return PairSet{b->prim64.ptr, b->prim32.ptr, b->pinfo.ptr, b->primdf.ptr, b->npairs, b->nprimpairs, b->primh.ptr,
+                 b->primhdf.ptr};
 }
 // Boys function of the reduced-precision (FP32) quartets: FP32 with
 // HF_JK_FP32_BOYS; else df64 in the df64 tier (the tier's stand-in for FP64);
@@ -185,7 +197,8 @@ inline PairSet hf_pairset(const hf_basis* b) {
 inline KernelCommon hf_kernel_common(const hf_ctx* c, unsigned jk_flags) {
   const int f32 = (jk_flags & HF_JK_FP32_BOYS) ? 1 : 0;
   const int df = (!f32 && (jk_flags & HF_JK_DF64)) ? 1 : 0;
-  return KernelCommon{c->boys64, c->boys32, f32, c->boysdf, df, 0, c->bounds, c->rys};  // det: set by hf_jk_run only
+  return KernelCommon{c->boys64, c->boys32, f32, c->boysdf, df, 0, c->bounds, c->rys,  // det: set by hf_jk_run only
+                      c->boysy64, c->boysydf};
 }
 // HF_JK_DETERMINISTIC is served by hf_fock_jk, hf_fock_jk_profiled and
 // hf_fock_jk_uhf; the entry points that build J/K elsewhere reject it.
@@ -246,5 +259,6 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
               const hf_jk_opts& o, cudaStream_t st, long long* nquartets, JKClassTiming* timing,
               const JKSpin* spin = nullptr);
 int hf_boys_tables(hf_ctx* ctx);
+void hf_boysy_fill(uint32_t* t64, uint32_t* tdf);  // the S_m(y) tables, boysy64_off(LMAX + 1) and boysydf_off(LMAX + 1) words
 int hf_eri_tensor_device(hf_basis* b, double* G);
 int hf_jk_stored_device(hf_basis* b, const double* G, const double* D, double* J, double* K);

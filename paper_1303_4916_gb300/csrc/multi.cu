@@ -63,7 +63,11 @@ int MultiJK::build(hf_ctx* c, const std::vector<hf_basis*>& mols, const std::vec
     t.active = 1;
     t.ps = hf_pairset(b);
     t.ketlist = b->ketlist.ptr;
-    for (int y = 0; y < HF_NPAIRCLASS; ++y) t.ket_off[y] = b->class_begin[y];
+    t.ketu = b->ketu.ptr;
+    for (int y = 0; y < HF_NPAIRCLASS; ++y) {
+      t.ket_off[y] = b->class_begin[y];
+      t.ketu_off[y] = b->ketu_begin[y];
+    }
   }
   HF_CHECK(table.alloc(ctx, std::max(nmol, 1)));
   if (nmol > 0)
@@ -89,9 +93,9 @@ int MultiJK::build(hf_ctx* c, const std::vector<hf_basis*>& mols, const std::vec
         hm.push_back(m);
         hs.push_back(nsp);
         hio.push_back((int)next);
-        nq += cnt;
-        mol_quartets[m] += cnt;
       }
+      nq += cw.nquartets;
+      mol_quartets[m] += cw.nquartets;
     }
     const int nb = (int)hb.size();
     HF_CHECK(bra[c2].alloc(ctx, nb));
@@ -111,6 +115,7 @@ int MultiJK::build(hf_ctx* c, const std::vector<hf_basis*>& mols, const std::vec
     JKWork& wk = w[c2];
     wk.bra = bra[c2].ptr;
     wk.ket = nullptr;
+    wk.ketu = nullptr;
     wk.kbeg = kbeg[c2].ptr;
     wk.kend = kend[c2].ptr;
     wk.ioff = ioff[c2].ptr;

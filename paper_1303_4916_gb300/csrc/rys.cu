@@ -732,7 +732,11 @@ __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const Pa
     const PairInfo bra = ps.info[bp];
     const bool add = it.nsp > (w.nchunk > 0 ? w.nchunk : 1);
     for (int kidx = it.k0; kidx < it.k1; ++kidx) {
-      const int kp = __ldg(w.ket + kidx);
+      // lists of ket units (the thread-per-quartet f/g classes): the quartet
+      // goes with its ket's first unit
+      const int2 unit = w.chunk == 32 ? __ldg(w.ketu + kidx) : make_int2(__ldg(w.ket + kidx), 0);
+      if ((unit.y >> 16) != 0) continue;
+      const int kp = unit.x;
       const PairInfo ket = ps.info[kp];
       int q_lo, q_hi, c_lo, c_hi;
       rys_part(rc, w, bra, ket, it.part, it.nsp, &q_lo, &q_hi, &c_lo, &c_hi);
