@@ -314,7 +314,7 @@ __device__ __forceinline__ void load_prim_df(const float* __restrict__ base, int
 // descending then y: d xy, xz, yz carry sqrt(3); f xyz sqrt(15), the
 // mixed ones sqrt(5); g x^2yz-type sqrt(35), x^2y^2-type sqrt(35/3),
 // x^3y-type sqrt(7); s, p and the axial components 1.
-__device__ __forceinline__ constexpr double comp_scale(int l, int c) {
+__host__ __device__ __forceinline__ constexpr double comp_scale(int l, int c) {
   return l == 2   ? ((c == 1 || c == 2 || c == 4) ? 1.7320508075688772935 : 1.0)
          : l == 3 ? (c == 4 ? 3.8729833462074168852 : (c == 0 || c == 6 || c == 9) ? 1.0 : 2.2360679774997896964)
          : l == 4 ? ((c == 0 || c == 10 || c == 14)  ? 1.0

@@ -22,6 +22,7 @@
 // and the operator's own centre C (the Hellmann-Feynman term), whose
 // derivative of (i|1/r_C|j) is -(d/dA + d/dB) by translational invariance,
 // takes -4 D_ij d(i|1/r_C|j)/dA.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -280,14 +281,32 @@ extern "C" int hf_rhf_gradient(hf_basis* b, const double* C, const double* eps, 
   HF_CUDA(cudaMemsetAsync(b->counters.ptr, 0, sizeof(int) * 2 * HF_NCLASS, st));
   const PairSet ps = hf_pairset(b);
   const KernelCommon kc = hf_kernel_common(ctx, 0);
-  for (int c = HF_NCLASS - 1; c >= 0; --c) {
+  // the classes run beside each other on the side streams (they share only
+  // the gradient's atomics), heaviest first
+  HF_CUDA(cudaEventRecord(ctx->fork_ev, st));
+  for (int k = 0; k < hf_ctx::kSide; ++k) HF_CUDA(cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
+  int nside = 0, rc = HF_OK;
+  for (int c = HF_NCLASS - 1; c >= 0 && rc == HF_OK; --c) {
     const ClassWork& cw = b->work64[c];
     if (cw.w.nitems <= 0) continue;
     JKWork w = cw.w;
     w.counter = b->counters.ptr + 2 * c;
+    int X = 0;
+    while ((X + 1) * (X + 2) / 2 <= c) ++X;
+    const int yb = b->class_begin[c - X * (X + 1) / 2];
+    double pq = 0.0;
+    for (int e = 0; e < w.nbra; ++e)  // primitive counts are uniform inside a bucket
+      pq += (double)b->nprim_sig_h[cw.bra_h[e]] * b->nprim_sig_h[b->ketlist_h[yb + cw.kbeg_h[e]]] *
+            (cw.kend_h[e] - cw.kbeg_h[e]);
     NvtxRange nv_cls(ctx->ops[c].name ? ctx->ops[c].name : "class");
-    ctx->ops[c].grad(w, ps, kc, D.ptr, bfa.ptr, n, g.ptr, 4 * ctx->num_sms, st);
+    rc = hf_grad_launch(ctx, c, w, ps, kc, D.ptr, bfa.ptr, n, g.ptr, pq * std::max(1, w.nchunk) / w.nitems,
+                        ctx->side[nside++ % hf_ctx::kSide]);
   }
+  for (int k = 0; k < hf_ctx::kSide; ++k) {  // joined also after a failed launch: the side work uses D and g
+    HF_CUDA(cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
+    HF_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[k], 0));
+  }
+  HF_CHECK(rc);
   HF_CUDA(cudaGetLastError());
   std::vector<double> gh(3 * (size_t)na);
   HF_CUDA(cudaMemcpyAsync(gh.data(), g.ptr, gh.size() * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -187,12 +187,6 @@ typedef void (*jk_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&,
 typedef void (*store_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&, double*, int, int, cudaStream_t);
 typedef void (*schwarz_launch_fn)(const int*, int, const PairSet&, const KernelCommon&, double*, cudaStream_t);
 typedef int (*occ_fn)();
-// Nuclear-gradient launch of one class: the class's Rys work list, the
-// density D (nbf x nbf), the atom of every basis function, and the
-// gradient accumulator (natom x 3).
-typedef void (*grad_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&, const double* D,
-                               const int* bf_atom, int nbf, double* grad, int grid, cudaStream_t);
-
 struct EriClassOps {
   jk_launch_fn jk64;
   jk_launch_fn jk32;
@@ -204,7 +198,6 @@ struct EriClassOps {
   occ_fn occ32;
   occ_fn occdf;
   occ_fn occrys;
-  grad_launch_fn grad;  // derivative ERIs contracted for the RHF gradient (Rys route, every class)
   int chunk;      // kets per work item: 32 (warp of quartets) or 1 (warp-cooperative class)
   int rys_nchunks;  // output chunks per quartet of the Rys kernel (every class)
   int rys_native;   // the class has an f or g shell: only the Rys kernel serves it

@@ -30,6 +30,7 @@ int hf_fail(int code, const char* fmt, ...);  // records the message, returns co
   } while (0)
 
 // ------------------------------------------------------------- context
+struct HfGradTabs;
 struct hf_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -44,6 +45,7 @@ struct hf_ctx {
   uint32_t* boysy64 = nullptr;  // S_m(y) of the Hermite kernels (hf_device.h)
   uint32_t* boysydf = nullptr;
   double* rys = nullptr;    // Rys roots and weights table (rys.cuh)
+  HfGradTabs* grad_tabs = nullptr;  // gradient class tables built so far (rys_grad.cu)
   EriClassOps ops[HF_NCLASS] = {};
   static constexpr int kSide = 8;
   cudaStream_t side[kSide] = {};     // class launches fork onto these
@@ -259,6 +261,9 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
               const hf_jk_opts& o, cudaStream_t st, long long* nquartets, JKClassTiming* timing,
               const JKSpin* spin = nullptr);
 int hf_boys_tables(hf_ctx* ctx);
+int hf_grad_launch(hf_ctx* ctx, int cls, const JKWork& w, const PairSet& ps, const KernelCommon& kc, const double* D,
+                   const int* bf_atom, int nbf, double* grad, double avg_pq, cudaStream_t st);
+void hf_grad_tabs_free(HfGradTabs* t);
 void hf_boysy_fill(uint32_t* t64, uint32_t* tdf);  // the S_m(y) tables, boysy64_off(LMAX + 1) and boysydf_off(LMAX + 1) words
 int hf_eri_tensor_device(hf_basis* b, double* G);
 int hf_jk_stored_device(hf_basis* b, const double* G, const double* D, double* J, double* K);
