@@ -38,6 +38,7 @@ extern "C" int hf_scf_solve_batch(hf_basis* const* bases, int count, const hf_sc
   cudaSetDevice(ctx->device);
   const auto t0 = std::chrono::steady_clock::now();
   std::vector<std::unique_ptr<ScfState>> S(count);
+  std::vector<ScfState*> Sp(count);
   std::vector<int> active(count, 0);
   std::vector<hf_basis*> mols(bases, bases + count);
   std::vector<const double*> Dp(count);
@@ -45,6 +46,7 @@ extern "C" int hf_scf_solve_batch(hf_basis* const* bases, int count, const hf_sc
   int first_error = HF_OK;
   for (int i = 0; i < count; ++i) {
     S[i].reset(new ScfState());
+    Sp[i] = S[i].get();
     int rc = hf_basis_prepare_work(mols[i], o.jk.schwarz_tau, o.jk.fp32_bound, o.jk.flags);
     if (rc == HF_OK) rc = scf_state_init(mols[i], *S[i], o.diis_size);
     if (rc == HF_OK) rc = scf_begin(mols[i], *S[i], o, nullptr);
@@ -66,8 +68,7 @@ extern "C" int hf_scf_solve_batch(hf_basis* const* bases, int count, const hf_sc
   for (int a : active) nactive += a;
   while (nactive > 0) {
     NvtxRange nv("scf iteration (batch)");
-    for (int i = 0; i < count; ++i)
-      if (active[i]) HF_CHECK(scf_density(mols[i], *S[i]));
+    HF_CHECK(scf_density_batch(ctx, count, mols.data(), Sp.data(), active.data()));
     if (!mj.tuned) {
       HF_CHECK(mj.tune_step(kc));   // iterations 1-3 time the candidate launch shapes
     } else {

@@ -220,7 +220,13 @@ int scf_state_init(hf_basis* b, ScfState& s, int diis_size) {
   return HF_OK;
 }
 
+// Library solver above HF_EIG_SINGLE (its GPU-wide kernels overtake one block
+// there), the block-per-matrix solver up to it.
 static int syevd(hf_ctx* ctx, ScfState& s, double* A, double* w) {
+  if (s.n <= HF_EIG_SINGLE) {
+    const EigJob j{A, w, s.n};
+    return hf_eig_small(ctx, &j, 1);
+  }
   if (cusolverDnDsyevd(ctx->cusolver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_LOWER, s.n, A, s.n, w, s.work.ptr,
                        s.lwork, s.info.ptr) != CUSOLVER_STATUS_SUCCESS)
     return hf_fail(HF_ERR_CUDA, "cusolverDnDsyevd failed");
@@ -259,19 +265,50 @@ int scf_setup(hf_basis* b, ScfState& s) {
 
 // Phase 1 of an iteration (enqueue only): from the current s.F,
 // F' = X F X, eigen-decomposition, C = X C', D = C_occ C_occ^T.
-int scf_density(hf_basis* b, ScfState& s) {
-  hf_ctx* ctx = b->ctx;
-  cudaStream_t st = ctx->stream;
-  const int n = s.n, nocc = b->nelec / 2;
-  const size_t nn = (size_t)n * n;
+static int density_before(hf_ctx* ctx, ScfState& s) {
+  const int n = s.n;
   HF_CHECK(gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, s.F.ptr, n, s.X.ptr, n, s.T1.ptr, n));
-  HF_CHECK(gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, s.X.ptr, n, s.T1.ptr, n, s.W.ptr, n));
-  HF_CHECK(syevd(ctx, s, s.W.ptr, s.eps.ptr));
+  return gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, s.X.ptr, n, s.T1.ptr, n, s.W.ptr, n);
+}
+
+static int density_after(hf_basis* b, ScfState& s) {
+  hf_ctx* ctx = b->ctx;
+  const int n = s.n, nocc = b->nelec / 2;
   HF_CHECK(gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, s.X.ptr, n, s.W.ptr, n, s.C.ptr, n));
   if (nocc > 0) {
     HF_CHECK(gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_T, n, n, nocc, s.C.ptr, n, s.C.ptr, n, s.D.ptr, n));
   } else {
-    HF_CUDA(cudaMemsetAsync(s.D.ptr, 0, nn * sizeof(double), st));
+    HF_CUDA(cudaMemsetAsync(s.D.ptr, 0, (size_t)n * n * sizeof(double), ctx->stream));
+  }
+  return HF_OK;
+}
+
+int scf_density(hf_basis* b, ScfState& s) {
+  HF_CHECK(density_before(b->ctx, s));
+  HF_CHECK(syevd(b->ctx, s, s.W.ptr, s.eps.ptr));
+  return density_after(b, s);
+}
+
+int scf_density_batch(hf_ctx* ctx, int count, hf_basis* const* b, ScfState* const* s, const int* active) {
+  // the blocks of one launch run side by side, so here the block-per-matrix
+  // solver pays up to the largest matrix it holds, given company
+  std::vector<EigJob> jobs;
+  std::vector<int> small(count, 0);
+  for (int i = 0; i < count; ++i)
+    if (active[i] && s[i]->n <= HF_EIG_NMAX) jobs.push_back(EigJob{s[i]->W.ptr, s[i]->eps.ptr, s[i]->n});
+  const int limit = jobs.size() > 1 ? HF_EIG_NMAX : HF_EIG_SINGLE;
+  jobs.clear();
+  for (int i = 0; i < count; ++i) {
+    if (!active[i]) continue;
+    HF_CHECK(density_before(ctx, *s[i]));
+    small[i] = s[i]->n <= limit;
+    if (small[i]) jobs.push_back(EigJob{s[i]->W.ptr, s[i]->eps.ptr, s[i]->n});
+  }
+  if (!jobs.empty()) HF_CHECK(hf_eig_small(ctx, jobs.data(), (int)jobs.size()));
+  for (int i = 0; i < count; ++i) {
+    if (!active[i]) continue;
+    if (!small[i]) HF_CHECK(syevd(ctx, *s[i], s[i]->W.ptr, s[i]->eps.ptr));
+    HF_CHECK(density_after(b[i], *s[i]));
   }
   return HF_OK;
 }

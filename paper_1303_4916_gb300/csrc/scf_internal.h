@@ -4,6 +4,19 @@
 
 #include "hf_internal.h"
 
+// One symmetric matrix (column-major, lower triangle read) to decompose:
+// on return its columns are the eigenvectors and w the ascending eigenvalues.
+struct EigJob {
+  double* A;
+  double* w;
+  int n;
+};
+#define HF_EIG_BATCH 32   // matrices per launch
+#define HF_EIG_NMAX 88    // three matrices in a block's shared memory
+#define HF_EIG_SINGLE 64
+// The block-per-matrix solver of eig.cu for every job (n <= HF_EIG_NMAX), on the context's stream.
+int hf_eig_small(hf_ctx* ctx, const EigJob* jobs, int count);
+
 struct ScfState {
   int n = 0, m = 0;
   DevArray<double> H, X, F, Fk, W, C, D, J, K, T1, T2, eps, scal, work, Fring, Ering, F1;
@@ -34,6 +47,9 @@ int scf_setup(hf_basis* b, ScfState& s);
 int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G);
 int scf_iterate(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G);
 int scf_density(hf_basis* b, ScfState& s);
+// the same for several molecules on one context (active[i] != 0), their
+// eigenproblems solved side by side
+int scf_density_batch(hf_ctx* ctx, int count, hf_basis* const* b, ScfState* const* s, const int* active);
 int scf_post_jk(hf_basis* b, ScfState& s);
 int scf_diis_step(hf_basis* b, ScfState& s);
 bool scf_after_iter(hf_basis* b, ScfState& s, const hf_scf_opts& o);

@@ -167,8 +167,16 @@ void hf_server::run() {
     }
     // one SCF iteration for every active molecule
     NvtxRange nv("serve round");
-    for (Request* r : active)
-      if (rc == HF_OK) rc = scf_density(r->basis, *r->scf);
+    if (rc == HF_OK) {
+      std::vector<hf_basis*> bs;
+      std::vector<ScfState*> ss;
+      for (Request* r : active) {
+        bs.push_back(r->basis);
+        ss.push_back(r->scf.get());
+      }
+      const std::vector<int> all(active.size(), 1);
+      rc = scf_density_batch(ctx, (int)active.size(), bs.data(), ss.data(), all.data());
+    }
     if (rc == HF_OK && !tuned) {
       rc = mj->tune_step(kc);       // the first rounds double as autotuner trials
       if (mj->tuned) {
