@@ -259,8 +259,8 @@ extern "C" int hf_rys_rule(int n, double T, double* u, double* w) {
 namespace hfr {
 
 // Fixed part of a warp's shared slice (doubles): transfer coefficients of
-// the bra [3][6][6] and the ket, roots, weights, component scales [4][21].
-constexpr int kCb = 0, kCd = 108, kRu = 216, kRw = 225, kSc = 240;  // kHead in all
+// the bra [3][6][6] and the ket, roots, weights; kHead in all.
+constexpr int kCb = 0, kCd = 108, kRu = 216, kRw = 225;
 
 __host__ __device__ inline int la1_(const RysClass& rc) { return rc.la + 1; }
 
@@ -293,40 +293,19 @@ struct Radix {
   }
 };
 
-__device__ __forceinline__ double dfact_odd(int x) {  // (2x-1)!!
-  double r = 1.0;
-  for (int k = 2 * x - 1; k > 1; k -= 2) r *= k;
-  return r;
-}
-
-// Per quartet: transfer coefficients C(b,k) AB^(b-k) (bra) and
-// C(d,k) CD^(d-k) (ket), and the component scales s(l, c) =
-// sqrt((2l-1)!! / ((2x-1)!! (2y-1)!! (2z-1)!!)) of the axial-normalised
-// basis.
-__device__ void rys_setup(const RysClass& rc, const double* AB, const double* CD, double* s, int lane) {
-  for (int e = lane; e < 2 * 108; e += 32) {
-    const int side = e / 108, r = e - side * 108;
-    const int dir = r / 36, ib = (r / 6) % 6, k = r % 6;
-    double v = 0.0;
-    if (k <= ib) {
-      double bin = 1.0;
-      for (int i = 1; i <= k; ++i) bin = bin * (ib - k + i) / i;
-      const double x = side ? CD[dir] : AB[dir];
-      double pw = 1.0;
-      for (int i = 0; i < ib - k; ++i) pw *= x;
-      v = bin * pw;
-    }
-    s[side ? kCd + r : kCb + r] = v;
-  }
-  for (int e = lane; e < 4 * 21; e += 32) {
-    const int sh = e / 21, c = e - sh * 21;
-    const int l = sh == 0 ? rc.la : sh == 1 ? rc.lb : sh == 2 ? rc.lc : rc.ld;
-    double v = 0.0;
-    if (c < (l + 1) * (l + 2) / 2) {
-      const int p = cart(l, c);
-      v = sqrt(dfact_odd(l) / (dfact_odd(p & 15) * dfact_odd((p >> 4) & 15) * dfact_odd(p >> 8)));
-    }
-    s[kSc + e] = v;
+// Per quartet: transfer coefficients C(b,k) AB^(b-k) (bra) and C(d,k)
+// CD^(d-k) (ket), for the powers the class has.
+__device__ __forceinline__ void rys_setup(const RysClass& rc, const double* AB, const double* CD, double* s, int lane) {
+  const int nb = 3 * (rc.lb + 1) * (rc.lb + 1), nd = 3 * (rc.ld + 1) * (rc.ld + 1);
+  for (int e = lane; e < nb + nd; e += 32) {
+    const bool ket = e >= nb;
+    const int l1 = (ket ? rc.ld : rc.lb) + 1, r = ket ? e - nb : e;
+    const int dir = r / (l1 * l1), t = r - dir * l1 * l1, ib = t / l1, k = t - ib * l1;
+    if (k > ib) continue;
+    const double x = ket ? (dir == 0 ? CD[0] : dir == 1 ? CD[1] : CD[2]) : (dir == 0 ? AB[0] : dir == 1 ? AB[1] : AB[2]);
+    double v = kBin.b[ib][k];
+    for (int i = 0; i < ib - k; ++i) v *= x;
+    s[(ket ? kCd : kCb) + (dir * 6 + ib) * 6 + k] = v;
   }
 }
 
@@ -470,7 +449,7 @@ __device__ void rys_rows(const RysClass& rc, const double* __restrict__ prim, co
       const int rl = e / NCD, cd = e - rl * NCD;
       const int row = r0 + rl, a = row / NB, b = row - a * NB;
       const int c = cd / ND, d = cd - c * ND;
-      blk[e] = acc[k] * s[kSc + a] * s[kSc + 21 + b] * s[kSc + 42 + c] * s[kSc + 63 + d];
+      blk[e] = acc[k] * (kBin.sc[rc.la][a] * kBin.sc[rc.lb][b] * kBin.sc[rc.lc][c] * kBin.sc[rc.ld][d]);
     }
   }
   __syncwarp();
@@ -694,7 +673,11 @@ void set_smem_attr_km() {
   switch ((rc).km) {             \
     case 4: F(4); break;         \
     case 8: F(8); break;         \
+    case 12: F(12); break;       \
     case 16: F(16); break;       \
+    case 20: F(20); break;       \
+    case 24: F(24); break;       \
+    case 28: F(28); break;       \
     default: F(32); break;       \
   }
 

@@ -4,6 +4,7 @@
 #pragma once
 #include <algorithm>
 
+#include "eri.cuh"
 #include "hf_device.h"
 #include "rys.cuh"
 
@@ -27,8 +28,26 @@ static __constant__ CartTable kCart = make_cart();
 
 __device__ __forceinline__ int cart(int l, int c) { return kCart.v[l * (l + 1) * (l + 2) / 6 + c]; }
 
+// Binomials, small integers and the component scales s(l, c) = sqrt((2l-1)!! /
+// ((2x-1)!! (2y-1)!! (2z-1)!!)) of the axial-normalised basis.
+struct BinTable {
+  double b[6][6];  // C(n, k)
+  double k[16];    // k as a double
+  double sc[5][15];
+};
+constexpr BinTable make_bin() {
+  BinTable t{};
+  for (int n = 0; n < 6; ++n)
+    for (int k = 0; k <= n; ++k) t.b[n][k] = hfk::binom_c(n, k);
+  for (int k = 0; k < 16; ++k) t.k[k] = k;
+  for (int l = 0; l < 5; ++l)
+    for (int c = 0; c < (l + 1) * (l + 2) / 2; ++c) t.sc[l][c] = hfk::comp_scale(l, c);
+  return t;
+}
+static __constant__ BinTable kBin = make_bin();
+
 // Fixed part of a warp's shared slice of the J/K kernels (doubles).
-constexpr int kHead = 328;
+constexpr int kHead = 234;
 
 // Outputs of one chunk: at most 32 per lane.
 constexpr int kMaxChunk = 1024;
@@ -71,10 +90,14 @@ inline RysClass rys_class(int la, int lb, int lc, int ld) {
   r.oI = ld == 0 ? r.oH : end;  // ld = 0: I is H
   if (ld > 0) end = r.oI + 3 * r.SI;
   const int ncd = r.nc * r.nd, rows = r.na * r.nb;
-  r.rpc = std::max(1, std::min(rows, kMaxChunk / ncd));
+  // as few chunks as fit, of even size: cutting off kMaxChunk at a time left
+  // (fd|dp), 60 rows of 18, a second chunk of 4 rows with tables of its own
+  const int most = std::max(1, std::min(rows, kMaxChunk / ncd));
+  const int least = (rows + most - 1) / most;
+  r.rpc = (rows + least - 1) / least;
   r.nchunks = (rows + r.rpc - 1) / r.rpc;
   const int per_lane = (r.rpc * ncd + 31) / 32;
-  r.km = per_lane <= 4 ? 4 : per_lane <= 8 ? 8 : per_lane <= 16 ? 16 : 32;
+  r.km = per_lane <= 4 ? 4 : per_lane <= 8 ? 8 : (per_lane + 3) / 4 * 4;
   r.native = std::max(std::max(la, lb), std::max(lc, ld)) > 2;
   r.oBlk = kHead;
   r.ws = (std::max(end, r.oBlk + r.rpc * ncd) + 1) & ~1;

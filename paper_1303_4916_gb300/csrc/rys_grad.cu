@@ -188,22 +188,6 @@ inline std::vector<uint32_t> grad_table(GradClass* gc) {
   return t;
 }
 
-struct BinTable {
-  double b[6][6];  // C(n, k)
-  double k[16];    // k as a double
-  double sc[5][15];
-};
-constexpr BinTable make_bin() {
-  BinTable t{};
-  for (int n = 0; n < 6; ++n)
-    for (int k = 0; k <= n; ++k) t.b[n][k] = hfk::binom_c(n, k);
-  for (int k = 0; k < 16; ++k) t.k[k] = k;
-  for (int l = 0; l < 5; ++l)
-    for (int c = 0; c < (l + 1) * (l + 2) / 2; ++c) t.sc[l][c] = hfk::comp_scale(l, c);
-  return t;
-}
-static __constant__ BinTable kBin = make_bin();
-
 // sum_k C(n, k) X^(n - k) f[k stride]
 __device__ __forceinline__ double move_power(const double* f, int stride, int n, double X) {
   double v = f[0];
