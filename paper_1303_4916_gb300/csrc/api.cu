@@ -201,6 +201,10 @@ int hf_boys_tables(hf_ctx* ctx) {
   HF_CHECK(hf_dev_alloc(ctx, &p, tyd.size() * sizeof(uint32_t)));
   ctx->boysydf = (uint32_t*)p;
   HF_CUDA(cudaMemcpyAsync(ctx->boysydf, tyd.data(), tyd.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
+  const std::vector<uint32_t> ct = hf_coop_tables();
+  HF_CHECK(hf_dev_alloc(ctx, &p, ct.size() * sizeof(uint32_t)));
+  ctx->cooptab = (uint32_t*)p;
+  HF_CUDA(cudaMemcpyAsync(ctx->cooptab, ct.data(), ct.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
   HF_CHECK(hf_dev_alloc(ctx, &p, ndf * sizeof(float)));
   ctx->boysdf = (float*)p;
   HF_CUDA(cudaMemcpyAsync(ctx->boysdf, tdf.data(), ndf * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
@@ -316,6 +320,7 @@ void hf_ctx_teardown(hf_ctx* c) {
   if (c->boysdf) hf_dev_free(c, c->boysdf, 0);
   if (c->boysy64) hf_dev_free(c, c->boysy64, 0);
   if (c->boysydf) hf_dev_free(c, c->boysydf, 0);
+  if (c->cooptab) hf_dev_free(c, c->cooptab, 0);
   if (c->rys) hf_dev_free(c, c->rys, 0);
   if (c->grad_tabs) hf_grad_tabs_free(c->grad_tabs);
   if (c->bounds) hf_dev_free(c, c->bounds, 0);

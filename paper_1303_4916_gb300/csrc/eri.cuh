@@ -26,7 +26,7 @@
 
 #include "df64.cuh"
 #include "eri_classes.cuh"
-#include "herm.cuh"
+#include "herm_coop.cuh"
 #include "hf_device.h"
 #include "rys.cuh"
 
@@ -712,7 +712,10 @@ struct CoopSizes {
   static constexpr int NAB = C::NA * C::NB, NCD = C::NC * C::ND;
   static constexpr int ROW = HF_NCOEF + C::L + 1;  // one primitive quartet's coefficients and B_m
   static constexpr int WS_HRR = NT + NAB * C::NF + NAB * NCD;
-  __host__ __device__ static constexpr int ws(int g) { return C::NSLOT + g * ROW > WS_HRR ? C::NSLOT + g * ROW : WS_HRR; }  // words per warp
+  __host__ __device__ static constexpr int ws(int g) { return C::NSLOT + g * ROW > WS_HRR ? C::NSLOT + g * ROW : WS_HRR; }  // words per warp (float)
+  static constexpr int WSH = CoopTab<C>::WS > WS_HRR ? CoopTab<C>::WS : WS_HRR;                  // (double, df64)
+  template <typename R>
+  __host__ __device__ static constexpr int words(int g) { return std::is_same<R, float>::value ? ws(g) : WSH; }
   // rows set up per pass: one per lane.  Measured on GB300 (60-atom s+p+d
   // molecule) 32 beats 16 and 8 in every class, (dd|dd) included although
   // its 124 KB per block then allow one block per SM: the serial part of
@@ -724,25 +727,18 @@ __device__ __forceinline__ double comp_scale_rt(int l, int c) {
   return (l == 2 && (c == 1 || c == 2 || c == 4)) ? 1.7320508075688772935 : 1.0;
 }
 
-// The contracted Cartesian block of one shell quartet (bra|ket) over its
-// primitive quartets [q_lo, q_hi), by one warp, in the scheme described
-// above; on return the warp's shared memory s holds it after the [e0|f0]
-// and the bra HRR rows: as doubles pre-multiplied by the d-component scales
-// (R = double or df64) or as floats (R = float), at s + NT + NAB * NF.
+// [e0|f0] of one shell quartet over its primitive quartets [q_lo, nq) by the
+// node list, in the scheme described above.
 template <class C, typename R, typename PB>
-__device__ __forceinline__ void coop_block(const PB* __restrict__ pbase, const KernelCommon& kc, const PairInfo& bra,
+__device__ __forceinline__ void coop_nodes(const PB* __restrict__ pbase, const KernelCommon& kc, const PairInfo& bra,
                                            const PairInfo& ket, int q_lo, int nq, R* const s, const int G,
-                                           const int lane) {
+                                           const int lane, R (&acc)[(C::NE * C::NF + 31) / 32]) {
   using S = CoopSizes<C>;
-  constexpr int NB = C::NB, NC = C::NC, ND = C::ND, NE = C::NE, NF = C::NF;
-  constexpr int NT = S::NT, NAB = S::NAB, NCD = S::NCD, NK = (NT + 31) / 32;
-  (void)NC;
-  (void)ND;
+  constexpr int NT = S::NT, NK = (NT + 31) / 32;
   R* const stage = s + C::NSLOT;
   const uint4* __restrict__ nodes = hfgen::CoopTables<C>::nodes();
   const int* __restrict__ levels = hfgen::CoopTables<C>::levels();
   const unsigned short* __restrict__ tgt = hfgen::CoopTables<C>::targets();
-  R acc[NK];
 #pragma unroll
   for (int k = 0; k < NK; ++k) acc[k] = (R)0;
   for (int g0 = q_lo; g0 < nq; g0 += G) {
@@ -810,16 +806,40 @@ __device__ __forceinline__ void coop_block(const PB* __restrict__ pbase, const K
       __syncwarp();
     }
   }
+}
+
+// The contracted Cartesian block of one shell quartet (bra|ket) over its
+// primitive quartets [q_lo, nq), by one warp: [e0|f0] by the Hermite form in
+// FP64 and df64, by the node list in FP32, then the HRR.  On return the warp's
+// shared memory s holds the block after the [e0|f0] and the bra HRR rows: as
+// doubles pre-multiplied by the d-component scales (R = double or df64) or as
+// floats (R = float), at s + NT + NAB * NF.
+template <class C, typename R>
+__device__ __forceinline__ void coop_block(const PairSet& P, const KernelCommon& kc, const PairInfo& bra,
+                                           const PairInfo& ket, int q_lo, int nq, R* const s, const int G,
+                                           const int lane) {
+  using S = CoopSizes<C>;
+  constexpr int NB = C::NB, NC = C::NC, ND = C::ND, NE = C::NE, NF = C::NF;
+  constexpr int NT = S::NT, NAB = S::NAB, NCD = S::NCD, NK = (NT + 31) / 32;
+  (void)NC;
+  (void)ND;
+  [[maybe_unused]] R acc[NK];
+  if constexpr (std::is_same<R, float>::value)
+    coop_nodes<C, R>(P.prim32, kc, bra, ket, q_lo, nq, s, G, lane, acc);
+  else
+    coop_herm<C, R>(P, kc, bra, ket, q_lo, nq, s, lane);  // leaves them at s
   // contracted [e0|f0] -> shared memory, then HRR
   R* const A = s;
   R* const H = s + NT;
   R* const I = H + NAB * NF;
   constexpr bool kPre = sizeof(R) == sizeof(double);      // R = double or df64
   double* const Id = reinterpret_cast<double*>(I);        // same storage when kPre
+  if constexpr (std::is_same<R, float>::value) {
 #pragma unroll
-  for (int k = 0; k < NK; ++k) {
-    const int tt = lane + 32 * k;
-    if (tt < NT) A[tt] = acc[k];
+    for (int k = 0; k < NK; ++k) {
+      const int tt = lane + 32 * k;
+      if (tt < NT) A[tt] = acc[k];
+    }
   }
   __syncwarp();
   {
@@ -864,9 +884,8 @@ __global__ void __launch_bounds__(128) eri_jk_coop_kernel(const JKWork w, const 
   constexpr int NB = C::NB, NC = C::NC, ND = C::ND, NE = C::NE, NF = C::NF;
   constexpr int NT = S::NT, NAB = S::NAB, NCD = S::NCD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* const s = reinterpret_cast<R*>(smem_raw) + (threadIdx.x >> 5) * S::ws(G);
+  R* const s = reinterpret_cast<R*>(smem_raw) + (threadIdx.x >> 5) * S::template words<R>(G);
   const int lane = threadIdx.x & 31;
-  const auto* base = PrimBase<R>::get(ps);
   for (;;) {
     int t = 0;
     if (lane == 0) t = atomicAdd(w.counter, 1);
@@ -881,7 +900,6 @@ __global__ void __launch_bounds__(128) eri_jk_coop_kernel(const JKWork w, const 
     const MolJK* mjp = mols ? mols + __ldg(w.mol + bi) : nullptr;
     if (mjp && !mjp->active) continue;
     const PairSet P = mjp ? mjp->ps : ps;
-    const auto* pbase = mjp ? PrimBase<R>::get(mjp->ps) : base;
     const int* ketb = mjp ? mjp->ketlist + mjp->ket_off[pair_class(C::LC, C::LD)] : w.ket;
     const int bp = __ldg(w.bra + bi);
     const int nsp = w.nsplit ? __ldg(w.nsplit + bi) : 1;
@@ -906,7 +924,7 @@ __global__ void __launch_bounds__(128) eri_jk_coop_kernel(const JKWork w, const 
     // parts' digested blocks add up)
     const int nq_all = bra.nprim * ket.nprim;
     const int q_lo = part * nq_all / nsp, nq = (part + 1) * nq_all / nsp;
-    coop_block<C, R>(pbase, kc, bra, ket, q_lo, nq, s, G, lane);
+    coop_block<C, R>(P, kc, bra, ket, q_lo, nq, s, G, lane);
     R* const I = s + NT + NAB * NF;
     constexpr bool kPre = sizeof(R) == sizeof(double);      // R = double or df64
     double* const Id = reinterpret_cast<double*>(I);        // same storage when kPre
@@ -1004,13 +1022,13 @@ __global__ void __launch_bounds__(128) eri_schwarz_coop_kernel(const int* __rest
   constexpr int NT = S::NT, NAB = S::NAB, NCD = S::NCD, NF = C::NF;
   static_assert(NAB == NCD, "diagonal class");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* const s = reinterpret_cast<double*>(smem_raw) + (threadIdx.x >> 5) * S::ws(G);
+  double* const s = reinterpret_cast<double*>(smem_raw) + (threadIdx.x >> 5) * S::WSH;
   const int lane = threadIdx.x & 31;
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one pair per warp
   if (t >= npairs) return;
   const int pid = pairs[t];
   const PairInfo pr = ps.info[pid];
-  coop_block<C, double>(ps.prim64, kc, pr, pr, 0, pr.nprim * pr.nprim, s, G, lane);
+  coop_block<C, double>(ps, kc, pr, pr, 0, pr.nprim * pr.nprim, s, G, lane);
   __syncwarp();
   const double* const Id = s + NT + NAB * NF;  // pre-scaled: (ab|ab) s_a^2 s_b^2
   double m = 0.0;
@@ -1034,7 +1052,7 @@ inline int coop_group() {
 
 template <class C, typename R>
 inline size_t coop_smem_bytes(int g) {
-  return (size_t)4 * CoopSizes<C>::ws(g) * sizeof(R);
+  return (size_t)4 * CoopSizes<C>::template words<R>(g) * sizeof(R);
 }
 
 template <class C, typename R>
@@ -1145,7 +1163,7 @@ __global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, con
   using S = CoopSizes<C>;
   constexpr int NB = C::NB, ND = C::ND, NF = C::NF, NAB = S::NAB, NCD = S::NCD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* const s = reinterpret_cast<double*>(smem_raw) + (threadIdx.x >> 5) * S::ws(g);
+  double* const s = reinterpret_cast<double*>(smem_raw) + (threadIdx.x >> 5) * S::WSH;
   const int lane = threadIdx.x & 31;
   for (;;) {
     int t = 0;
@@ -1165,7 +1183,7 @@ __global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, con
     const PairInfo bra = ps.info[bp];
     const PairInfo ket = ps.info[kp];
     const int nq = bra.nprim * ket.nprim;
-    coop_block<C, double>(ps.prim64, kc, bra, ket, part * nq / nsp, (part + 1) * nq / nsp, s, g, lane);
+    coop_block<C, double>(ps, kc, bra, ket, part * nq / nsp, (part + 1) * nq / nsp, s, g, lane);
     __syncwarp();
     const double* const Id = s + S::NT + NAB * NF;  // scaled by the d components
     const size_t n = (size_t)nbf;

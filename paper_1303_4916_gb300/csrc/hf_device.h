@@ -31,7 +31,7 @@
 // large-argument form, at y_i = i / 8, i = 256 .. 1024.  A FP64 row holds
 // S_0..S_L as doubles, S_1..S_{L+3} as (hi, lo) float pairs and S_{L+4..L+6}
 // as floats; a df64 row S_0..S_{L+3} as pairs and S_{L+4..L+7} as floats.
-#define BOYSY_LMAX 4
+#define BOYSY_LMAX 8
 #define BOYSY64_NNEAR 3841
 #define BOYSYDF_NNEAR 961
 #define BOYSY_NFAR 769
@@ -119,6 +119,7 @@ struct KernelCommon {
   const double* rys;  // Rys roots and weights table (rys.cuh layout)
   const unsigned* boysy64;  // S_m(y) tables of the Hermite kernels
   const unsigned* boysydf;
+  const uint32_t* cooptab;  // index tables of the warp-cooperative Hermite kernels (coop_tab.cu)
 };
 
 // Bounds-checked build (-DHF_BOUNDS_CHECK, small cases in place of a memory

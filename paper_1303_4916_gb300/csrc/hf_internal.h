@@ -44,6 +44,7 @@ struct hf_ctx {
   float* boysdf = nullptr;
   uint32_t* boysy64 = nullptr;  // S_m(y) of the Hermite kernels (hf_device.h)
   uint32_t* boysydf = nullptr;
+  uint32_t* cooptab = nullptr;  // index tables of herm_coop.cuh
   double* rys = nullptr;    // Rys roots and weights table (rys.cuh)
   HfGradTabs* grad_tabs = nullptr;  // gradient class tables built so far (rys_grad.cu)
   EriClassOps ops[HF_NCLASS] = {};
@@ -200,7 +201,7 @@ inline KernelCommon hf_kernel_common(const hf_ctx* c, unsigned jk_flags) {
   const int f32 = (jk_flags & HF_JK_FP32_BOYS) ? 1 : 0;
   const int df = (!f32 && (jk_flags & HF_JK_DF64)) ? 1 : 0;
   return KernelCommon{c->boys64, c->boys32, f32, c->boysdf, df, 0, c->bounds, c->rys,  // det: set by hf_jk_run only
-                      c->boysy64, c->boysydf};
+                      c->boysy64, c->boysydf, c->cooptab};
 }
 // HF_JK_DETERMINISTIC is served by hf_fock_jk, hf_fock_jk_profiled and
 // hf_fock_jk_uhf; the entry points that build J/K elsewhere reject it.
@@ -264,6 +265,7 @@ int hf_boys_tables(hf_ctx* ctx);
 int hf_grad_launch(hf_ctx* ctx, int cls, const JKWork& w, const PairSet& ps, const KernelCommon& kc, const double* D,
                    const int* bf_atom, int nbf, double* grad, double avg_pq, cudaStream_t st);
 void hf_grad_tabs_free(HfGradTabs* t);
+std::vector<uint32_t> hf_coop_tables();
 void hf_boysy_fill(uint32_t* t64, uint32_t* tdf);  // the S_m(y) tables, boysy64_off(LMAX + 1) and boysydf_off(LMAX + 1) words
 int hf_eri_tensor_device(hf_basis* b, double* G);
 int hf_jk_stored_device(hf_basis* b, const double* G, const double* D, double* J, double* K);
