@@ -204,10 +204,31 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
       next = t;
     });
   };
-  // H and the left-over X of n quartets, coefficients from ck on
+  // H and the left-over X of n quartets, coefficients from ck on.  Both passes
+  // go through one copy of the unrolled sums (they change places in between):
+  // two copies of the df64 code overran the instruction cache (issue active
+  // 13 % in (dd|dd), 25 % in (dd|dp), waiting for instructions).
   auto add_terms = [&](const R* ck, int n) {
-    for (int j = sm; j < n; j += T::PM) herm_terms_add<C, R>(s + T::oR + j * T::NR, ck + j * T::NCK, pm, H);
-    if (T::TL > 0 && sl < n) herm_terms_add<C, R>(s + T::oR + sl * T::NR, ck + sl * T::NCK, pl, X);
+#pragma unroll 1
+    for (int ps = 0; ps < (T::TL > 0 ? 2 : 1); ++ps) {
+#pragma unroll 1
+      for (int j = ps ? sl : sm; j < n; j += ps ? 32 : T::PM)
+        herm_terms_add<C, R>(s + T::oR + j * T::NR, ck + j * T::NCK, pm, H);
+      if constexpr (T::TL > 0) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          const R t = H[f];
+          H[f] = X[f];
+          X[f] = t;
+        }
+#pragma unroll
+        for (int k = 0; k < T::NUW; ++k) {
+          const uint32_t t = pm[k];
+          pm[k] = pl[k];
+          pl[k] = t;
+        }
+      }
+    }
   };
   auto clear = [&]() {
 #pragma unroll
