@@ -15,10 +15,6 @@
 #include "multi.h"
 #include "scf_internal.h"
 
-int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G);
-bool scf_after_iter(hf_basis* b, ScfState& s, const hf_scf_opts& o);
-int scf_finish(hf_basis* b, ScfState& s, hf_scf_result* r);
-
 extern "C" int hf_scf_solve_batch(hf_basis* const* bases, int count, const hf_scf_opts* opts, hf_scf_result* results,
                                   int* status) {
   if (!bases || !results || !status || count <= 0) return hf_fail(HF_ERR_INVALID, "hf_scf_solve_batch: bad arguments");
@@ -49,7 +45,13 @@ extern "C" int hf_scf_solve_batch(hf_basis* const* bases, int count, const hf_sc
     Sp[i] = S[i].get();
     int rc = hf_basis_prepare_work(mols[i], o.jk.schwarz_tau, o.jk.fp32_bound, o.jk.flags);
     if (rc == HF_OK) rc = scf_state_init(mols[i], *S[i], o.diis_size);
-    if (rc == HF_OK) rc = scf_begin(mols[i], *S[i], o, nullptr);
+    status[i] = rc;
+    if (rc == HF_ERR_CUDA) return rc;
+  }
+  HF_CHECK(scf_setup_batch(ctx, count, mols.data(), Sp.data(), status));
+  for (int i = 0; i < count; ++i) {
+    int rc = status[i];
+    if (rc == HF_OK) rc = scf_begin(mols[i], *S[i], o, nullptr, true);
     status[i] = rc;
     active[i] = rc == HF_OK;
     if (rc != HF_OK && first_error == HF_OK) first_error = rc;

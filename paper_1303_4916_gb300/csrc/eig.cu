@@ -60,10 +60,9 @@ __device__ __forceinline__ void rotation(float app, float aqq, float apq, float*
   *s = t * *c;
 }
 __device__ __forceinline__ void rotation(double app, double aqq, double apq, double* c, double* s) {
-  // the ratio decides the angle: differences are formed in FP64, and the
-  // scale (elements far below the FP32 range) divided out
-  const double d = aqq - app, a = fmax(fabs(d), fabs(apq)), f = a > 0.0 ? 1.0 / a : 0.0;
-  const double t = (double)jacobi_t(0.0f, (float)(d * f), (float)(apq * f));
+  // the difference is formed in FP64; the matrix is scaled to elements of at
+  // most 1, so FP32 holds what is worth rotating (above 2^-55)
+  const double t = (double)jacobi_t(0.0f, (float)(aqq - app), (float)apq);
   *c = hfk::hf_rsqrt(fma(t, t, 1.0));
   *s = t * *c;
 }
@@ -190,13 +189,15 @@ __global__ void __launch_bounds__(kThreads) eig_kernel(const EigBatch batch) {
   __syncthreads();
   mx = red[0];
   for (int k = 1; k < kThreads / 32; ++k) mx = fmax(mx, red[k]);
-  const double scale = mx > 0.0 ? 1.0 / mx : 1.0;
+  // scaled by a power of two (exactly) to elements in [-1, 1]
+  const int ex = mx > 0.0 && mx < 1e300 ? ilogb(mx) + 1 : 0;
+  const double down = scalbn(1.0, -ex), up = scalbn(1.0, ex);
   auto el = [&](int i, int j) -> double {
-    return i < n && j < n ? A[(size_t)min(i, j) * n + max(i, j)] : 0.0;
+    return i < n && j < n ? A[(size_t)min(i, j) * n + max(i, j)] * down : 0.0;
   };
   for (int t = tid; t < m * m; t += kThreads) {
     const int i = t / m, j = t - i * m;
-    B[i * ld + j] = (float)(el(i, j) * scale);
+    B[i * ld + j] = (float)el(i, j);
     V[i * ld + j] = i == j ? 1.0f : 0.0f;
   }
   __syncthreads();
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kThreads) eig_kernel(const EigBatch batch) {
   __syncthreads();
   small_gemm(S1, 1, ld, S2, S0, m, ld, true, [](double v, int, int) { return v; });
   __syncthreads();
-  jacobi<double>(S0, S1, m, ld, cs, cs + m / 2, mx * 0x1p-55, 16);
+  jacobi<double>(S0, S1, m, ld, cs, cs + m / 2, 0x1p-55, 16);
   // ascending order; the pad (a zero row, never rotated into the others) goes last
   for (int i = tid; i < n; i += kThreads) {
     const double w = S0[i * ld + i];
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(kThreads) eig_kernel(const EigBatch batch) {
       const double x = S0[j * ld + j];
       rank += x < w || (x == w && j < i);
     }
-    job.w[rank] = w;
+    job.w[rank] = w * up;
     cs[i] = (double)rank;
   }
   __syncthreads();

@@ -241,16 +241,22 @@ static int gemm(hf_ctx* ctx, cublasOperation_t ta, cublasOperation_t tb, int m, 
   return HF_OK;
 }
 
-// H = T + V and X = S^{-1/2}; fills s.smin.
-int scf_setup(hf_basis* b, ScfState& s) {
+// H = T + V and X = S^{-1/2}; fills s.smin.  In three parts, so that a batch's
+// overlap matrices are decomposed side by side.
+static int setup_before(hf_basis* b, ScfState& s) {
+  hf_ctx* ctx = b->ctx;
+  const size_t nn = (size_t)s.n * s.n;
+  HF_CHECK(hf_basis_one_electron(b));
+  k_add<<<blocks(nn), 256, 0, ctx->stream>>>(b->T.ptr, b->V.ptr, s.H.ptr, nn);
+  HF_CUDA(cudaMemcpyAsync(s.W.ptr, b->S.ptr, nn * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
+  return HF_OK;
+}
+
+static int setup_after(hf_basis* b, ScfState& s) {
   hf_ctx* ctx = b->ctx;
   cudaStream_t st = ctx->stream;
   const int n = s.n;
   const size_t nn = (size_t)n * n;
-  HF_CHECK(hf_basis_one_electron(b));
-  k_add<<<blocks(nn), 256, 0, st>>>(b->T.ptr, b->V.ptr, s.H.ptr, nn);
-  HF_CUDA(cudaMemcpyAsync(s.W.ptr, b->S.ptr, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  HF_CHECK(syevd(ctx, s, s.W.ptr, s.eps.ptr));
   double smin = 0.0;
   HF_CUDA(cudaMemcpyAsync(&smin, s.eps.ptr, sizeof(double), cudaMemcpyDeviceToHost, st));
   HF_CUDA(cudaStreamSynchronize(st));
@@ -259,7 +265,40 @@ int scf_setup(hf_basis* b, ScfState& s) {
   // X = (U s^{-1/2}) U^T
   HF_CUDA(cudaMemcpyAsync(s.T1.ptr, s.W.ptr, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
   k_scale_cols<<<blocks(nn), 256, 0, st>>>(s.T1.ptr, s.eps.ptr, n);
-  HF_CHECK(gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_T, n, n, n, s.T1.ptr, n, s.W.ptr, n, s.X.ptr, n));
+  return gemm(ctx, CUBLAS_OP_N, CUBLAS_OP_T, n, n, n, s.T1.ptr, n, s.W.ptr, n, s.X.ptr, n);
+}
+
+int scf_setup(hf_basis* b, ScfState& s) {
+  HF_CHECK(setup_before(b, s));
+  HF_CHECK(syevd(b->ctx, s, s.W.ptr, s.eps.ptr));
+  return setup_after(b, s);
+}
+
+// The eigenproblems W -> (W, eps) of the states with active[i] != 0, the small
+// ones side by side: the blocks of one launch run on different SMs, so here
+// the block-per-matrix solver pays up to the largest matrix it holds, given
+// company.
+static int syevd_batch(hf_ctx* ctx, int count, ScfState* const* s, const int* active) {
+  std::vector<EigJob> jobs;
+  for (int i = 0; i < count; ++i)
+    if (active[i] && s[i]->n <= HF_EIG_NMAX) jobs.push_back(EigJob{s[i]->W.ptr, s[i]->eps.ptr, s[i]->n});
+  const int limit = jobs.size() > 1 ? HF_EIG_NMAX : HF_EIG_SINGLE;
+  jobs.erase(std::remove_if(jobs.begin(), jobs.end(), [&](const EigJob& j) { return j.n > limit; }), jobs.end());
+  if (!jobs.empty()) HF_CHECK(hf_eig_small(ctx, jobs.data(), (int)jobs.size()));
+  for (int i = 0; i < count; ++i)
+    if (active[i] && s[i]->n > limit) HF_CHECK(syevd(ctx, *s[i], s[i]->W.ptr, s[i]->eps.ptr));
+  return HF_OK;
+}
+
+int scf_setup_batch(hf_ctx* ctx, int count, hf_basis* const* b, ScfState* const* s, int* status) {
+  std::vector<int> live(count);
+  for (int i = 0; i < count; ++i) {
+    if (status[i] == HF_OK) status[i] = setup_before(b[i], *s[i]);
+    live[i] = status[i] == HF_OK;
+  }
+  HF_CHECK(syevd_batch(ctx, count, s, live.data()));
+  for (int i = 0; i < count; ++i)
+    if (live[i]) status[i] = setup_after(b[i], *s[i]);
   return HF_OK;
 }
 
@@ -290,26 +329,11 @@ int scf_density(hf_basis* b, ScfState& s) {
 }
 
 int scf_density_batch(hf_ctx* ctx, int count, hf_basis* const* b, ScfState* const* s, const int* active) {
-  // the blocks of one launch run side by side, so here the block-per-matrix
-  // solver pays up to the largest matrix it holds, given company
-  std::vector<EigJob> jobs;
-  std::vector<int> small(count, 0);
   for (int i = 0; i < count; ++i)
-    if (active[i] && s[i]->n <= HF_EIG_NMAX) jobs.push_back(EigJob{s[i]->W.ptr, s[i]->eps.ptr, s[i]->n});
-  const int limit = jobs.size() > 1 ? HF_EIG_NMAX : HF_EIG_SINGLE;
-  jobs.clear();
-  for (int i = 0; i < count; ++i) {
-    if (!active[i]) continue;
-    HF_CHECK(density_before(ctx, *s[i]));
-    small[i] = s[i]->n <= limit;
-    if (small[i]) jobs.push_back(EigJob{s[i]->W.ptr, s[i]->eps.ptr, s[i]->n});
-  }
-  if (!jobs.empty()) HF_CHECK(hf_eig_small(ctx, jobs.data(), (int)jobs.size()));
-  for (int i = 0; i < count; ++i) {
-    if (!active[i]) continue;
-    if (!small[i]) HF_CHECK(syevd(ctx, *s[i], s[i]->W.ptr, s[i]->eps.ptr));
-    HF_CHECK(density_after(b[i], *s[i]));
-  }
+    if (active[i]) HF_CHECK(density_before(ctx, *s[i]));
+  HF_CHECK(syevd_batch(ctx, count, s, active));
+  for (int i = 0; i < count; ++i)
+    if (active[i]) HF_CHECK(density_after(b[i], *s[i]));
   return HF_OK;
 }
 
@@ -444,11 +468,11 @@ int scf_finish(hf_basis* b, ScfState& s, hf_scf_result* r) {
   return HF_OK;
 }
 
-int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G) {
+int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G, bool set_up) {
   hf_ctx* ctx = b->ctx;
   cudaStream_t st = ctx->stream;
   const size_t nn = (size_t)s.n * s.n;
-  HF_CHECK(scf_setup(b, s));
+  if (!set_up) HF_CHECK(scf_setup(b, s));
   s.iter = 0;
   s.converged = 0;
   s.energy = 0.0;

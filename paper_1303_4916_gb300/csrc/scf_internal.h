@@ -44,7 +44,10 @@ struct ScfState {
 
 int scf_state_init(hf_basis* b, ScfState& s, int diis_size);
 int scf_setup(hf_basis* b, ScfState& s);
-int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G);
+// set_up: scf_setup or scf_setup_batch has been done
+int scf_begin(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G, bool set_up = false);
+// scf_setup of the states whose status[i] is HF_OK; each keeps its own status
+int scf_setup_batch(hf_ctx* ctx, int count, hf_basis* const* b, ScfState* const* s, int* status);
 int scf_iterate(hf_basis* b, ScfState& s, const hf_scf_opts& o, const double* G);
 int scf_density(hf_basis* b, ScfState& s);
 // the same for several molecules on one context (active[i] != 0), their
