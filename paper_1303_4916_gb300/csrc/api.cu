@@ -111,7 +111,7 @@ void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
   };
   long double F[BOYS_NM], et;
   auto rows = [&](uint32_t* t, int nrow0, bool df) {  // S_m in F -> row nrow0 of every slice
-    for (int L = 0; L <= BOYSY_LMAX; ++L) {
+    for (int L = df ? 1 : 0; L <= BOYSY_LMAX; ++L) {
       uint32_t* r = t + (df ? boysydf_off(L) + (size_t)nrow0 * BOYSYDF_ROW(L) : boysy64_off(L) + (size_t)nrow0 * BOYSY64_ROW(L));
       if (!df)
         for (int m = 0; m <= L; ++m, r += 2) {
@@ -129,19 +129,33 @@ void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
       }
     }
   };
-  for (int i = 0; i < BOYSY64_NNEAR; ++i) {
-    boys_row((long double)i / 64.0L, F, &et);
+  auto row0 = [&](int row) {  // the df64 row of L = 0
+    uint32_t* r = tdf + (size_t)row * BOYSYDF_ROW(0);
+    for (int m = 0; m < 3; ++m) {
+      float q[2];
+      split(F[m], q);
+      memcpy(r + 2 * m, q, sizeof q);
+    }
+    for (int m = 3; m < 5; ++m) {
+      const float v = (float)F[m];
+      memcpy(r + 3 + m, &v, sizeof v);
+    }
+  };
+  for (int i = 0; i < BOYSYDF0_NNEAR; ++i) {
+    boys_row((long double)i / 128.0L, F, &et);
     for (int m = 1; m < BOYS_NM; m += 2) F[m] = -F[m];
-    rows(t64, i, false);
-    if (i % 4 == 0) rows(tdf, i / 4, true);
+    row0(i);
+    if (i % 2 == 0) rows(t64, i / 2, false);
+    if (i % 8 == 0) rows(tdf, i / 8, true);
   }
   const long double pi = 3.141592653589793238462643383279502884L;
-  for (int i = 0; i < BOYSY_NFAR; ++i) {
-    const long double T = (256 + i) / 16.0L;
+  for (int i = 0; i < BOYSYDF0_NFAR; ++i) {
+    const long double T = (1024 + i) / 64.0L;
     F[0] = 0.5L * sqrtl(pi / T);
     for (int m = 1; m < BOYS_NM; ++m) F[m] = -F[m - 1] * (2 * m - 1) / (2.0L * T);
-    rows(t64, BOYSY64_NNEAR + i, false);
-    rows(tdf, BOYSYDF_NNEAR + i, true);
+    row0(BOYSYDF0_NNEAR + i);
+    if (i % 4 == 0) rows(t64, BOYSY64_NNEAR + i / 4, false);
+    if (i % 4 == 0) rows(tdf, BOYSYDF_NNEAR + i / 4, true);
   }
 }
 

@@ -179,11 +179,31 @@ __device__ __forceinline__ void boys_y(double y, const KernelCommon& kc, double*
 // size, since here the row loads are a larger share of the time.
 template <int L>
 __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) {
-  constexpr int ROW = BOYSYDF_ROW(L), F0 = 2 * (L + 4);
   const bool far = y.hi >= 120.0f;
   const int k = far ? ((__float_as_int(y.hi) >> 23) - 132) >> 1 : 0;
   const float sc = pow2f(-2 * k);
   const float yh = y.hi * sc, yl = y.lo * sc;  // exact
+  if constexpr (L == 0) {
+    // (ss|ss) is bound by L1 (each lane's row is a wavefront of its own), so
+    // its row is one 32-byte load on a finer grid (|z| <= 2^-8, far 2^-7 with
+    // T >= 16): terms to S_4
+    const float gs = far ? 32.0f : 64.0f;
+    const int i = __float2int_rn(yh * gs);
+    const float xh = __fsub_rn(yh, (float)i * (far ? 1.0f / 32.0f : 1.0f / 64.0f));  // exact (Sterbenz)
+    const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl);
+    unsigned r[8];
+    ldg256u(kc.boysydf + (size_t)(far ? i + (BOYSYDF0_NNEAR - 1024) : i) * 8, r);
+    auto w = [&](int j) { return __uint_as_float(r[j]); };
+    const float g = __fmaf_rn(w(7), z.hi * 0.25f, w(6));
+    df64 f = df_quick_two_sum(w(4), __fmaf_rn(g, z.hi * (1.0f / 3.0f), w(5)));
+    f = df_fma_small(f, df64(0.5f * z.hi, 0.5f * z.lo), df64(w(2), w(3)));
+    f = df_fma_small(f, z, df64(w(0), w(1)));
+    f = df_quick_two_sum(f.hi, f.lo);
+    const float s = pow2f(-k);
+    S[0] = df64(f.hi * s, f.lo * s);
+    return;
+  }
+  constexpr int ROW = BOYSYDF_ROW(L), F0 = 2 * (L + 4);
   const int i = __float2int_rn(yh * 8.0f);
   const float xh = __fsub_rn(yh, (float)i * 0.125f);  // exact (Sterbenz)
   const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl), z3 = third(z);

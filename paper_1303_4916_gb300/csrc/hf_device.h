@@ -35,13 +35,19 @@
 #define BOYSY64_NNEAR 3841
 #define BOYSYDF_NNEAR 961
 #define BOYSY_NFAR 769
+// df64, L = 0: rows of one 32-byte load (S_0, S_1, S_2 as pairs, S_3, S_4) on
+// a finer grid, near y_i = i / 64, far y_i = i / 32, i = 1024 .. 4096
+#define BOYSYDF0_NNEAR 7681
+#define BOYSYDF0_NFAR 3073
 #define BOYSY64_ROW(L) ((4 * (L) + 11 + 7) / 8 * 8)
-#define BOYSYDF_ROW(L) ((2 * (L) + 12 + 7) / 8 * 8)
+#define BOYSYDF_ROW(L) ((L) == 0 ? 8 : (2 * (L) + 12 + 7) / 8 * 8)
 __host__ __device__ constexpr size_t boysy64_off(int L) {
   return L == 0 ? 0 : boysy64_off(L - 1) + (size_t)(BOYSY64_NNEAR + BOYSY_NFAR) * BOYSY64_ROW(L - 1);
 }
 __host__ __device__ constexpr size_t boysydf_off(int L) {
-  return L == 0 ? 0 : boysydf_off(L - 1) + (size_t)(BOYSYDF_NNEAR + BOYSY_NFAR) * BOYSYDF_ROW(L - 1);
+  return L == 0   ? 0
+         : L == 1 ? (size_t)(BOYSYDF0_NNEAR + BOYSYDF0_NFAR) * BOYSYDF_ROW(0)
+                  : boysydf_off(L - 1) + (size_t)(BOYSYDF_NNEAR + BOYSY_NFAR) * BOYSYDF_ROW(L - 1);
 }
 // thread-per-quartet classes with L = la+lb+lc+ld up to this have a df64
 // variant; the warp-cooperative classes (L >= 5) take df64 through the
