@@ -176,27 +176,18 @@ __global__ void finish_fixed(const unsigned long long* __restrict__ Jq, const un
 // and the units of a class are split into as few buckets of neighbouring
 // sizes as give the least lane time, sum over buckets of ceil(n / 32) times
 // the largest size.  A cap of 12 costs a digestion per 12 primitives of a
-// long ket; a basis so small that its primitive quartets do not fill the GPU
-// takes a lower one, down to 3, to have more units.
-static void build_ket_units(hf_basis* b) {
+// long ket; lower ones (3, 5, 9) measured the same from 8 atoms (43 us) to 15.
+static void build_ket_units(hf_basis* b, const std::vector<int>& by_q) {
   const int np = b->npairs;
-  long long total = 0;
-  for (int k = 0; k < np; ++k) total += b->nprim_sig_h[k];
-  const double per_warp = (double)total * total / 64.0 / (16.0 * b->ctx->num_sms);  // lane steps of a whole build
-  const int cap = (int)std::min(12.0, std::max(3.0, per_warp));
-  b->qrank.assign(np, 0);
+  constexpr int cap = 12;
   b->ketu_h.clear();
   for (int X = 0; X < HF_NPAIRCLASS; ++X) {
     const int s0 = b->class_begin[X], s1 = b->class_begin[X + 1];
     b->ketu_begin[X] = (int)b->ketu_h.size();
     b->ubuckets[X].clear();
-    std::vector<int> by_q(s1 - s0);
-    std::iota(by_q.begin(), by_q.end(), s0);
-    std::stable_sort(by_q.begin(), by_q.end(), [&](int x, int y) { return b->Q_h[x] > b->Q_h[y]; });
     long long count[13] = {};
     for (int r = 0; r < s1 - s0; ++r) {
-      b->qrank[by_q[r]] = r;
-      const int n = b->nprim_sig_h[by_q[r]], nu = std::max(1, (n + cap - 1) / cap);
+      const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
       for (int u = 0; u < nu; ++u) ++count[(u + 1) * n / nu - u * n / nu];
     }
     // least lane time over the ways to cut sizes 0..12 into neighbouring
@@ -221,10 +212,10 @@ static void build_ket_units(hf_basis* b) {
     b->ubuckets[X].push_back(0);
     for (int z = 13; z > 0; z = cut[z]) {
       for (int r = 0; r < s1 - s0; ++r) {
-        const int n = b->nprim_sig_h[by_q[r]], nu = std::max(1, (n + cap - 1) / cap);
+        const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
         for (int u = 0; u < nu; ++u) {
           const int k0 = u * n / nu, k1 = (u + 1) * n / nu;
-          if (k1 - k0 >= cut[z] && k1 - k0 < z) b->ketu_h.push_back(make_int2(by_q[r], k0 << 16 | (k1 - k0)));
+          if (k1 - k0 >= cut[z] && k1 - k0 < z) b->ketu_h.push_back(make_int2(by_q[s0 + r], k0 << 16 | (k1 - k0)));
         }
       }
       const int end = (int)b->ketu_h.size() - b->ketu_begin[X];
@@ -234,6 +225,8 @@ static void build_ket_units(hf_basis* b) {
   // the pairs whole, in the order of the pair list: the FP32 ranges (an FP32
   // sum cut in other places rounds differently)
   b->ketw_begin = (int)b->ketu_h.size();
+  b->ketu_first.assign(1, 0);
+  for (const int2& u : b->ketu_h) b->ketu_first.push_back(b->ketu_first.back() + ((u.y >> 16) == 0));
   for (int k = 0; k < np; ++k) b->ketu_h.push_back(make_int2(b->ketlist_h[k], b->nprim_sig_h[b->ketlist_h[k]]));
 }
 
@@ -436,20 +429,28 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
     // the 32 lanes of a warp loop over the same number of primitives and
     // the Schwarz-surviving kets of a bucket are a prefix of it.
     b->ketlist_h.resize(np);
+    b->qrank.assign(np, 0);
+    std::vector<int> by_q(np), at(HF_MAX_NPRIM * HF_MAX_NPRIM + 2);
+    std::iota(by_q.begin(), by_q.end(), 0);
     for (int X = 0; X < HF_NPAIRCLASS; ++X) {
       const int s0 = b->class_begin[X], s1 = b->class_begin[X + 1];
-      for (int k = s0; k < s1; ++k) b->ketlist_h[k] = k;
-      std::stable_sort(b->ketlist_h.begin() + s0, b->ketlist_h.begin() + s1, [&](int x, int y) {
-        if (b->nprim_sig_h[x] != b->nprim_sig_h[y]) return b->nprim_sig_h[x] > b->nprim_sig_h[y];
-        return b->Q_h[x] > b->Q_h[y];
-      });
+      std::stable_sort(by_q.begin() + s0, by_q.begin() + s1, [&](int x, int y) { return b->Q_h[x] > b->Q_h[y]; });
+      // then stably by primitive count, descending (counting sort)
+      std::fill(at.begin(), at.end(), 0);
+      const int top = HF_MAX_NPRIM * HF_MAX_NPRIM;
+      for (int k = s0; k < s1; ++k) ++at[top - b->nprim_sig_h[by_q[k]] + 1];
+      for (int c = 1; c <= top + 1; ++c) at[c] += at[c - 1];
+      for (int k = s0; k < s1; ++k) {
+        b->qrank[by_q[k]] = k - s0;
+        b->ketlist_h[s0 + at[top - b->nprim_sig_h[by_q[k]]]++] = by_q[k];
+      }
       b->buckets[X].clear();
       for (int k = s0; k < s1; ++k)
         if (k == s0 || b->nprim_sig_h[b->ketlist_h[k]] != b->nprim_sig_h[b->ketlist_h[k - 1]])
           b->buckets[X].push_back(k - s0);
       b->buckets[X].push_back(s1 - s0);
     }
-    build_ket_units(b);
+    build_ket_units(b, by_q);
     if ((rc = b->ketu.alloc(ctx, b->ketu_h.size()))) break;
     if (cudaMemcpyAsync(b->ketlist.ptr, b->ketlist_h.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st) !=
             cudaSuccess ||
@@ -567,10 +568,8 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
             kb[r].push_back(lo + shift);
             ke[r].push_back(hi + shift);
             kprim[r].push_back(bucket_prims[u]);
-            if (units)  // a quartet counts with the first of its units
-              for (int k = lo; k < hi; ++k) nq[r] += (b->ketu_h[ub + k].y >> 16) == 0;
-            else
-              nq[r] += hi - lo;
+            // a quartet counts with the first of its units
+            nq[r] += units ? b->ketu_first[ub + hi] - b->ketu_first[ub + lo] : hi - lo;
           }
         }
       }
@@ -593,7 +592,7 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
           work += len[e] * ((ke[r][e] - kb[r][e] + chunk - 1) / chunk) * std::max(1, nchunk);
         }
         const long long warps = 16LL * ctx->num_sms;
-        const long long floor_len = rys_list ? 16 : chunk == 1 ? 64 : r == 0 ? 6 : 16;
+        const long long floor_len = rys_list ? 16 : chunk == 1 ? 64 : r == 0 ? 9 : 16;
         const long long target = std::max(floor_len, work / std::max(1LL, warps));
         sp[r].resize(ne);
         for (size_t e = 0; e < ne; ++e) {

@@ -158,6 +158,7 @@ struct hf_basis {
   // ket units of the 32-ket lists (JKWork::ketu), per pair class in buckets of like size, Q descending
   DevArray<int2> ketu;
   std::vector<int2> ketu_h;
+  std::vector<int> ketu_first;        // units before each position that are their pair's first
   int ketu_begin[HF_NPAIRCLASS] = {};
   int ketw_begin = 0;                 // then the pairs whole, in ketlist order
   std::vector<int> ubuckets[HF_NPAIRCLASS];
