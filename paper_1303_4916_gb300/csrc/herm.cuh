@@ -17,15 +17,15 @@
 //    w = rs^2 = 2 rho and y = w |PQ|^2 = 2 T, (-2 rho)^m F_m(T) =
 //    w^m S_m(y), S_m(y) = (-1)^m F_m(y / 2); the remaining sqrt(1 / (pq)) is
 //    in the records' prefactors.
-//  * 1/sqrt is the hardware estimate and one third-order correction, five
+//  * 1/sqrt is the hardware estimate and one third-order correction, four
 //    FP64 instructions (hf_rsqrt).
 //  * S_m is a tabulated FP64 value plus a Taylor tail of at most 2^-7 of it,
 //    evaluated in double-float arithmetic (48 bits) on the FP32 pipe: two
 //    FP64 additions per order instead of an eight-term FP64 Horner.  The tail
 //    contributes below 2^-54 of the value to its error.  The table index and
 //    the offset come from the bits of y, without FP64 conversions.
-// (ps|ss), FP64: 0.0508 ns per primitive quartet on the whole GPU, from 0.0996
-// (the pipe's rate is 629e9 FP64 instructions x lanes per second: 32 of them,
+// (ps|ss), FP64: 0.0489 ns per primitive quartet on the whole GPU, from 0.0996
+// (the pipe's rate is 629e9 FP64 instructions x lanes per second: 31 of them,
 // from 63).
 #pragma once
 #include <type_traits>
@@ -76,13 +76,23 @@ __device__ __forceinline__ df64 times_int(df64 a, int k) { return df_mulf(a, (fl
 __device__ __forceinline__ double fmah(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ df64 fmah(df64 a, df64 b, df64 c) { return df_fma(a, b, c); }
 
-// 1/sqrt(a), a normal and positive: the hardware estimate y0 (about 20 bits,
-// so y0^2 is exact) and the binomial series of (1 - e)^(-1/2), e = 1 - a y0^2,
-// to second order in e; the neglected 5/16 e^3 is below 2^-57.
+// y^2 for a positive normal y whose low word is zero, exact: the square of the
+// 21-bit significand in integers, so no FP64 instruction
+__device__ __forceinline__ double square_high(double y) {
+  const unsigned h = (unsigned)__double2hiint(y), m = (h & 0xfffffu) | 0x100000u;
+  const unsigned long long q = (unsigned long long)m * m;  // in [2^40, 2^42)
+  const int up = (int)(q >> 41);                           // 1: at least 2^41
+  const unsigned long long f = q << (12 - up);             // in [2^52, 2^53)
+  return __longlong_as_double((long long)(((unsigned long long)(2 * (int)(h >> 20) - 1024 + up) << 52) + f));
+}
+
+// 1/sqrt(a), a normal and positive: the hardware estimate y0 (its low word is
+// zero: 21 bits) and the binomial series of (1 - e)^(-1/2), e = 1 - a y0^2, to
+// second order in e; the neglected 5/16 e^3 is below 2^-57.
 __device__ __forceinline__ double hf_rsqrt(double a) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-a, y * y, 1.0);
+  const double e = fma(-a, square_high(y), 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ df64 hf_rsqrt(df64 a) { return rsqrt(a); }
@@ -338,7 +348,8 @@ __device__ __forceinline__ void contracted_herm(const PairSet& ps, const KernelC
       if constexpr (L == 0) {
         H[0] = fmah(g, B[0], H[0]);
       } else {
-        B[0] = g * B[0];
+        if constexpr (LK == 0) H[0] = fmah(g, B[0], H[0]);  // R_000 goes nowhere else
+        else B[0] = g * B[0];
 #pragma unroll
         for (int m = 1; m <= L; ++m) {
           g = g * w;
@@ -348,7 +359,7 @@ __device__ __forceinline__ void contracted_herm(const PairSet& ps, const KernelC
         herm_r<L>(B, PQ, r);
         if constexpr (LK == 0) {
 #pragma unroll
-          for (int t = 0; t < NT; ++t) H[t] = H[t] + r[t];
+          for (int t = 1; t < NT; ++t) H[t] = H[t] + r[t];
         } else {
           R e[3][LK + 1][LK + 1];
 #pragma unroll
