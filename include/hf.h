@@ -104,7 +104,7 @@ typedef struct {
                                       arithmetic, ~1e-14 relative, in every class (J/K
                                       digestion and accumulation stay FP64) */
 #define HF_JK_RYS 16u              /* every class by Rys quadrature (Eq. 5, the paper's route) in
-                                      FP64, in place of the Obara-Saika / Head-Gordon-Pople
+                                      FP64, in place of the Hermite and Obara-Saika
                                       kernels of the s/p/d classes; classes with an f or g shell
                                       always take it (in FP64 also under HF_JK_DF64 and for
                                       quartets below fp32_bound) */

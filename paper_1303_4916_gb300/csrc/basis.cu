@@ -36,9 +36,8 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
                             const int* __restrict__ sh_l, const int* __restrict__ sh_nprim,
                             const int* __restrict__ sh_prim, const int* __restrict__ sh_bf,
                             const double* __restrict__ exps, const double* __restrict__ coefs,
-                            double* __restrict__ prim64, float* __restrict__ prim32, float* __restrict__ primdf,
-                            double* __restrict__ primh, float* __restrict__ primhdf,
-                            PairInfo* __restrict__ info, double eps) {
+                            double* __restrict__ prim64, float* __restrict__ prim32,
+                            float* __restrict__ primdf, PairInfo* __restrict__ info, double eps) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npairs) return;
   const int A = pA[t], B = pB[t];
@@ -79,26 +78,18 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
                      pow(kPi, 1.25) / p;
     const double Px = (a * Ax + b * Bx) / p, Py = (a * Ay + b * By) / p, Pz = (a * Az + b * Bz) / p;
     double* r = prim64 + (size_t)(base + s) * PRIM64_STRIDE;
-    r[0] = p; r[1] = 0.5 / p; r[2] = Px; r[3] = Py; r[4] = Pz;
-    r[5] = Px - Ax; r[6] = Py - Ay; r[7] = Pz - Az; r[8] = K; r[9] = a;
+    r[0] = 0.5 / p; r[1] = Px; r[2] = Py; r[3] = Pz;
+    r[4] = Px - Ax; r[5] = Py - Ay; r[6] = Pz - Az; r[7] = K * 1.1892071150027210667 * sqrt(r[0]);
+    r[8] = p; r[9] = K; r[10] = a; r[11] = 0.0;
     float* f = prim32 + (size_t)(base + s) * PRIM32_STRIDE;
-    for (int x = 0; x < 10; ++x) f[x] = (float)r[x];
-    f[10] = 0.f; f[11] = 0.f;
+    f[0] = (float)p;
+    for (int x = 0; x < 7; ++x) f[1 + x] = (float)r[x];
+    f[8] = (float)K; f[9] = (float)a; f[10] = 0.f; f[11] = 0.f;
     float* g = primdf + (size_t)(base + s) * PRIMDF_STRIDE;
-    for (int x = 0; x < 10; ++x) {
+    for (int x = 0; x < 8; ++x) {
       const float h = __double2float_rn(r[x]);
       g[2 * x] = h;
       g[2 * x + 1] = __double2float_rn(r[x] - (double)h);
-    }
-    // record of the Hermite kernels: K'' = K 2^(1/4) (2p)^(-1/2)
-    double* rh = primh + (size_t)(base + s) * PRIMH_STRIDE;
-    float* gh = primhdf + (size_t)(base + s) * 2 * PRIMH_STRIDE;
-    const double hv[PRIMH_STRIDE] = {r[1], Px, Py, Pz, r[5], r[6], r[7], K * 1.1892071150027210667 * sqrt(r[1])};
-    for (int x = 0; x < PRIMH_STRIDE; ++x) {
-      rh[x] = hv[x];
-      const float h = __double2float_rn(hv[x]);
-      gh[2 * x] = h;
-      gh[2 * x + 1] = __double2float_rn(hv[x] - (double)h);
     }
   }
   PairInfo pi;
@@ -371,9 +362,7 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
         (rc = dbf.alloc(ctx, nshell + 1)) || (rc = dxyz.alloc(ctx, 3 * nshell)) || (rc = dexp.alloc(ctx, nprim)) ||
         (rc = dcoef.alloc(ctx, nprim)) || (rc = b->prim64.alloc(ctx, (size_t)off * PRIM64_STRIDE)) ||
         (rc = b->prim32.alloc(ctx, (size_t)off * PRIM32_STRIDE)) ||
-        (rc = b->primdf.alloc(ctx, (size_t)off * PRIMDF_STRIDE)) ||
-        (rc = b->primh.alloc(ctx, (size_t)off * PRIMH_STRIDE)) ||
-        (rc = b->primhdf.alloc(ctx, (size_t)off * 2 * PRIMH_STRIDE)) || (rc = b->pinfo.alloc(ctx, np)) ||
+        (rc = b->primdf.alloc(ctx, (size_t)off * PRIMDF_STRIDE)) || (rc = b->pinfo.alloc(ctx, np)) ||
         (rc = b->Q.alloc(ctx, np)) || (rc = b->ketlist.alloc(ctx, np)) || (rc = b->counters.alloc(ctx, 2 * HF_NCLASS)))
       break;
 #define UP(dst, src, cnt)                                                                                      \
@@ -393,8 +382,7 @@ extern "C" int hf_basis_create(hf_ctx* ctx, const hf_atom* atoms, int natom, con
     UP(dcoef, b->coefs.data(), nprim);
 #undef UP
     pair_kernel<<<(np + 127) / 128, 128, 0, st>>>(np, dA.ptr, dB.ptr, dOff.ptr, dxyz.ptr, dl.ptr, dn.ptr, dp.ptr, dbf.ptr,
-                                                  dexp.ptr, dcoef.ptr, b->prim64.ptr, b->prim32.ptr, b->primdf.ptr, b->primh.ptr,
-                                                  b->primhdf.ptr,
+                                                  dexp.ptr, dcoef.ptr, b->prim64.ptr, b->prim32.ptr, b->primdf.ptr,
                                                   b->pinfo.ptr, kPrimEps);
     if (cudaGetLastError() != cudaSuccess) { rc = hf_fail(HF_ERR_CUDA, "pair_kernel launch"); break; }
     // Schwarz factors per pair class, using the (X|X) diagonal quartets.
@@ -484,7 +472,7 @@ extern "C" int hf_basis_nshell(const hf_basis* b) { return b ? b->nshell : 0; }
 
 extern "C" size_t hf_basis_device_bytes(const hf_basis* b) {
   if (!b) return 0;
-  size_t s = b->prim64.bytes() + b->prim32.bytes() + b->primdf.bytes() + b->primh.bytes() + b->primhdf.bytes() + b->ketu.bytes() + b->pinfo.bytes() + b->Q.bytes() + b->ketlist.bytes() +
+  size_t s = b->prim64.bytes() + b->prim32.bytes() + b->primdf.bytes() + b->ketu.bytes() + b->pinfo.bytes() + b->Q.bytes() + b->ketlist.bytes() +
              b->counters.bytes() + b->hD.bytes() + b->hJ.bytes() + b->hK.bytes() + b->Dsum.bytes() + b->detq.bytes() + b->bfshell.bytes() + b->pairkey.bytes() + b->S.bytes() + b->T.bytes() +
              b->V.bytes();
   for (int c = 0; c < HF_NCLASS; ++c)
@@ -751,12 +739,13 @@ int hf_jk_run(hf_basis* b, const double* D, double* Jp, double* Kp, double* J, d
       }
     }
   }
-  HF_CUDA(cudaGetLastError());
-  if (fork)
+  const cudaError_t launched = cudaGetLastError();
+  if (fork)  // joined whatever the launches said: the side work uses the caller's buffers
     for (int k = 0; k < nuse; ++k) {
       HF_CUDA(cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
       HF_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[k], 0));
     }
+  HF_CUDA(launched);
   double* K2 = spin ? spin->K2 : nullptr;
   if (det)
     finish_fixed<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(q, q + 2 * nn, spin ? q + 4 * nn : nullptr, J, K, K2,
@@ -1010,11 +999,12 @@ int hf_eri_tensor_device(hf_basis* b, double* G) {
     if (w.w.nitems > 0)
       ctx->ops[c].store(w.w, ps, kc, G, n, hf_launch_grid(ctx, 4, w.w.nitems), ctx->side[nside++ % hf_ctx::kSide]);
   }
-  HF_CUDA(cudaGetLastError());
+  const cudaError_t launched = cudaGetLastError();
   for (int k = 0; k < hf_ctx::kSide; ++k) {
     HF_CUDA(cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
     HF_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[k], 0));
   }
+  HF_CUDA(launched);
   const unsigned chunks = (unsigned)std::min<size_t>(std::max<size_t>(1, nn / 1024), 16);
   mirror_tensor<<<dim3((unsigned)nn, chunks), 256, 0, st>>>(G, n, b->bfshell.ptr, b->pairkey.ptr, ns);
   HF_CUDA(cudaGetLastError());

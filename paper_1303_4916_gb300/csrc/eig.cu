@@ -17,8 +17,8 @@
 // below 2^-55 of the largest element of A, whatever the FP32 stage left
 // (clusters that FP32 cannot separate only take more FP64 rotations).
 // GB300: 0.74 ms for a 42 x 42 Fock matrix (library 1.6 ms in 45 launches); ten RHF
-// iterations of a 7-atom molecule from set-up 28.3 -> 19.0 ms, of six molecules of 4
-// to 9 atoms in a batch 115 -> 53 ms.
+// iterations of a 7-atom molecule from set-up 28.3 -> 17.8 ms, of six molecules of 4
+// to 9 atoms in a batch 115 -> 44.6 ms, the overlap matrices' solves included.
 #include <algorithm>
 
 #include "herm.cuh"

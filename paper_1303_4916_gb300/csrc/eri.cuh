@@ -1,12 +1,12 @@
 // eri.cuh -- per-class ERI kernels with the fused J/K contraction.
 //
-// One thread evaluates one contracted shell quartet (ab|cd) of Eq. 5; the
-// 32 lanes of a warp share the bra pair (ab) and take 32 consecutive kets
-// (cd) from the Schwarz-sorted ket list.  Per primitive quartet the thread
-// evaluates the Boys function F_m(T), m = 0..L, and the Obara-Saika VRR
-// (generated per class), accumulating [e0|f0]; after the primitive loop the
-// HRR gives the Cartesian block, which is digested straight into J and K
-// (the J/K equation of Sec. "Technical details").
+// One thread evaluates one contracted shell quartet (ab|cd) of Eq. 5 (or a
+// ket unit of it); the 32 lanes of a warp share the bra pair (ab) and take 32
+// consecutive kets from the Schwarz-sorted ket list.  The contracted [e0|f0]
+// comes from herm.cuh (FP64: bra in Hermite Gaussians; df64: Obara-Saika VRR
+// with the same set-up) or, for the FP32 ranges, from the VRR below; the HRR
+// gives the Cartesian block, which is digested straight into J and K (the J/K
+// equation of Sec. "Technical details").
 //
 // Digestion of one unique quartet with block I_abcd and degeneracy weight
 // w = 1 / |stabiliser| (1/2 for each of A==B, C==D, (AB)==(CD)):
@@ -125,13 +125,6 @@ struct Prim {
   R p, o2p, P[3], PA[3], K;
 };
 
-__device__ __forceinline__ void load_prim(const double* __restrict__ base, int idx, Prim<double>& q) {
-  const double2* s = reinterpret_cast<const double2*>(base + (size_t)idx * PRIM64_STRIDE);
-  const double2 a = __ldg(s), b = __ldg(s + 1), c = __ldg(s + 2), d = __ldg(s + 3), e = __ldg(s + 4);
-  q.p = a.x; q.o2p = a.y; q.P[0] = b.x; q.P[1] = b.y; q.P[2] = c.x;
-  q.PA[0] = c.y; q.PA[1] = d.x; q.PA[2] = d.y; q.K = e.x;
-}
-
 __device__ __forceinline__ void load_prim(const float* __restrict__ base, int idx, Prim<float>& q) {
   const float4* s = reinterpret_cast<const float4*>(base + (size_t)idx * PRIM32_STRIDE);
   const float4 a = __ldg(s), b = __ldg(s + 1), c = __ldg(s + 2);
@@ -139,28 +132,14 @@ __device__ __forceinline__ void load_prim(const float* __restrict__ base, int id
   q.PA[0] = b.y; q.PA[1] = b.z; q.PA[2] = b.w; q.K = c.x;
 }
 
-template <typename R> struct PrimBase;
-template <> struct PrimBase<double> { static __device__ __forceinline__ const double* get(const PairSet& s) { return s.prim64; } };
-template <> struct PrimBase<float> { static __device__ __forceinline__ const float* get(const PairSet& s) { return s.prim32; } };
-
-template <int L, typename R>
-struct BoysSel {
-  static __device__ __forceinline__ void eval(R T, const KernelCommon& kc, R* F);
-};
-template <int L>
-struct BoysSel<L, double> {
-  static __device__ __forceinline__ void eval(double T, const KernelCommon& kc, double* F) {
-    boys64<L>(T, kc.boys64, F);
-  }
-};
 template <int L>
 __device__ __forceinline__ void boys_df(df64 T, const float* __restrict__ tab, df64* F);
 
+// F_m of the reduced-precision quartets: in FP64 (table + downward recursion),
+// rounded to FP32 for the recurrences; in df64 (same recursion, 48-bit
+// significand) in the df64 tier; in FP32 when boys_fp32 is set.
 template <int L>
-struct BoysSel<L, float> {
-  // Reduced-precision quartets: F_m in FP64 (table + downward recursion),
-  // rounded to FP32 for the recurrences; in df64 (same recursion, 48-bit
-  // significand) in the df64 tier; in FP32 when boys_fp32 is set.
+struct BoysFloat {
   static __device__ __forceinline__ void eval(float T, const KernelCommon& kc, float* F) {
     if (kc.boys_fp32) {
       boys32<L>(T, kc.boys32, F);
@@ -178,13 +157,14 @@ struct BoysSel<L, float> {
   }
 };
 
-// Contracted block of one shell quartet: loops over the significant
-// primitive pairs of bra and ket.  nb/nk are the primitive-pair counts
+// Contracted [e0|f0] of one shell quartet in FP32 (the reduced-precision
+// ranges): loops over the significant primitive pairs of bra and ket.  nb/nk are the primitive-pair counts
 // (0 for an inactive lane).
-template <class C, typename R>
+template <class C>
 __device__ __forceinline__ void contracted_vrr(const PairSet& ps, const KernelCommon& kc, int b0, int nb,
-                                               int k0, int nk, R* acc) {
-  const auto* base = PrimBase<R>::get(ps);
+                                               int k0, int nk, float* acc) {
+  using R = float;
+  const float* base = ps.prim32;
 #pragma unroll
   for (int x = 0; x < C::NE * C::NF; ++x) acc[x] = (R)0;
   // ket primitives outer (a different record per lane, loaded once each),
@@ -196,7 +176,7 @@ __device__ __forceinline__ void contracted_vrr(const PairSet& ps, const KernelCo
       Prim<R> a;
       load_prim(base, b0 + ib, a);
       const R pq = a.p + c.p;
-      const R rs = (R)rsqrt(pq);
+      const R rs = rsqrt(pq);
       const R inv = rs * rs;
       const R rp = c.p * inv;  // rho / zeta
       const R rq = a.p * inv;  // rho / eta
@@ -209,7 +189,7 @@ __device__ __forceinline__ void contracted_vrr(const PairSet& ps, const KernelCo
       }
       const R T = a.p * rp * (PQ[0] * PQ[0] + PQ[1] * PQ[1] + PQ[2] * PQ[2]);
       R B[C::L + 1];
-      BoysSel<C::L, R>::eval(T, kc, B);
+      BoysFloat<C::L>::eval(T, kc, B);
       const R pref = a.K * c.K * rs;
 #pragma unroll
       for (int m = 0; m <= C::L; ++m) B[m] *= pref;
@@ -300,15 +280,6 @@ __device__ __forceinline__ void boys_df(df64 T, const float* __restrict__ tab, d
   }
 }
 
-__device__ __forceinline__ void load_prim_df(const float* __restrict__ base, int idx, Prim<df64>& q) {
-  const float4* s = reinterpret_cast<const float4*>(base + (size_t)idx * PRIMDF_STRIDE);
-  const float4 a = __ldg(s), b = __ldg(s + 1), c = __ldg(s + 2), d = __ldg(s + 3), e = __ldg(s + 4);
-  q.p = df64(a.x, a.y); q.o2p = df64(a.z, a.w);
-  q.P[0] = df64(b.x, b.y); q.P[1] = df64(b.z, b.w); q.P[2] = df64(c.x, c.y);
-  q.PA[0] = df64(c.z, c.w); q.PA[1] = df64(d.x, d.y); q.PA[2] = df64(d.z, d.w);
-  q.K = df64(e.x, e.y);
-}
-
 // Cartesian component scale relative to the axial component,
 // sqrt((2l-1)!! / ((2x-1)!! (2y-1)!! (2z-1)!!)), components ordered x power
 // descending then y: d xy, xz, yz carry sqrt(3); f xyz sqrt(15), the
@@ -375,18 +346,18 @@ __device__ __forceinline__ void rys_thread_block(const PairSet& P, const KernelC
   }
   for (int ib = ib0; ib < ib1; ++ib) {
     const double* rb = P.prim64 + (size_t)(bra.prim0 + ib) * PRIM64_STRIDE;
-    const double p = __ldg(rb), hp = __ldg(rb + 1);
-    const double Pp[3] = {__ldg(rb + 2), __ldg(rb + 3), __ldg(rb + 4)};
-    const double PA[3] = {__ldg(rb + 5), __ldg(rb + 6), __ldg(rb + 7)};
-    const double Kab = __ldg(rb + 8);
+    const double p = __ldg(rb + 8), hp = __ldg(rb);
+    const double Pp[3] = {__ldg(rb + 1), __ldg(rb + 2), __ldg(rb + 3)};
+    const double PA[3] = {__ldg(rb + 4), __ldg(rb + 5), __ldg(rb + 6)};
+    const double Kab = __ldg(rb + 9);
     for (int ik = 0; ik < nk; ++ik) {
       const double* rk = P.prim64 + (size_t)(k0 + ik) * PRIM64_STRIDE;
-      const double q = __ldg(rk), hq = __ldg(rk + 1);
-      const double PQ[3] = {Pp[0] - __ldg(rk + 2), Pp[1] - __ldg(rk + 3), Pp[2] - __ldg(rk + 4)};
-      const double QC[3] = {__ldg(rk + 5), __ldg(rk + 6), __ldg(rk + 7)};
+      const double q = __ldg(rk + 8), hq = __ldg(rk);
+      const double PQ[3] = {Pp[0] - __ldg(rk + 1), Pp[1] - __ldg(rk + 2), Pp[2] - __ldg(rk + 3)};
+      const double QC[3] = {__ldg(rk + 4), __ldg(rk + 5), __ldg(rk + 6)};
       const double ipq = 1.0 / (p + q);
       const double T = p * q * ipq * (PQ[0] * PQ[0] + PQ[1] * PQ[1] + PQ[2] * PQ[2]);
-      const double pref = Kab * __ldg(rk + 8) * sqrt(ipq);
+      const double pref = Kab * __ldg(rk + 9) * sqrt(ipq);
       const double qf = q * ipq, pf = p * ipq;
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
@@ -544,7 +515,7 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
     } else {
       R acc[C::NE * C::NF];
       if constexpr (std::is_same<R, float>::value)
-        contracted_vrr<C, R>(P, kc, bra.prim0 + ib0, ib1 - ib0, k0, nk, acc);
+        contracted_vrr<C>(P, kc, bra.prim0 + ib0, ib1 - ib0, k0, nk, acc);
       else
         contracted<C, R>(P, kc, bra.prim0 + ib0, ib1 - ib0, k0, nk, acc);
       R AB[3] = {(R)bra.AB[0], (R)bra.AB[1], (R)bra.AB[2]};
@@ -679,22 +650,14 @@ __global__ void __launch_bounds__(128) eri_jk_kernel(const JKWork w, const PairS
 }
 
 // ------------------------------------------------------------- cooperative kernel
-// df64 hooks of the generic (cooperative) kernel
-__device__ __forceinline__ void load_prim(const float* __restrict__ base, int idx, Prim<df64>& q) {
-  load_prim_df(base, idx, q);
-}
-template <> struct PrimBase<df64> { static __device__ __forceinline__ const float* get(const PairSet& s) { return s.primdf; } };
-template <int L>
-struct BoysSel<L, df64> {
-  static __device__ __forceinline__ void eval(df64 T, const KernelCommon& kc, df64* F) { boys_df<L>(T, kc.boysdf, F); }
-};
-
 // a * b + c, fused in each arithmetic type of the cooperative kernel (the
 // df64 one sits beside df_fma, where argument-dependent lookup finds it)
 __device__ __forceinline__ double fmac(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fmac(float a, float b, float c) { return fmaf(a, b, c); }
 
-// Classes with L >= 5: one warp per contracted quartet.  The primitive
+// Classes with L >= 5: one warp per contracted quartet.  In FP64 and df64 the
+// contracted [e0|f0] come from coop_herm (herm_coop.cuh).  In FP32 (the
+// FP32 split's ranges) from node lists (coop_nodes): the primitive
 // quartets are set up G at a time, one per lane: each lane forms its
 // coefficient vector (PA, WP, QC, WQ, rho/p, rho/q, k/(2p), k/(2q),
 // k/(2(p+q))) and B_m = prefactor * F_m in a row of shared memory.  The
@@ -702,8 +665,8 @@ __device__ __forceinline__ float fmac(float a, float b, float c) { return fmaf(a
 // lanes evaluate the generated VRR node list level by level (node =
 // c0 x0 + c1 x1 [+ c2 (x2 - c3 x3)] [+ c4 x4] over slots, c from the row,
 // the bracketed terms as the node's type bits say), and
-// lane l adds the targets l, l+32, ... into its registers.  After the
-// primitive loop the contracted [e0|f0] go to shared memory, the bra HRR
+// lane l adds the targets l, l+32, ... into its registers.  After either
+// primitive loop the contracted [e0|f0] are in shared memory, the bra HRR
 // runs one f per lane, the ket HRR one ab per lane, and each of the six
 // digestion contractions gives one output element per lane.
 template <class C>
@@ -728,11 +691,12 @@ __device__ __forceinline__ double comp_scale_rt(int l, int c) {
 }
 
 // [e0|f0] of one shell quartet over its primitive quartets [q_lo, nq) by the
-// node list, in the scheme described above.
-template <class C, typename R, typename PB>
-__device__ __forceinline__ void coop_nodes(const PB* __restrict__ pbase, const KernelCommon& kc, const PairInfo& bra,
-                                           const PairInfo& ket, int q_lo, int nq, R* const s, const int G,
-                                           const int lane, R (&acc)[(C::NE * C::NF + 31) / 32]) {
+// node list, in the scheme described above, in FP32.
+template <class C>
+__device__ __forceinline__ void coop_nodes(const float* __restrict__ pbase, const KernelCommon& kc, const PairInfo& bra,
+                                           const PairInfo& ket, int q_lo, int nq, float* const s, const int G,
+                                           const int lane, float (&acc)[(C::NE * C::NF + 31) / 32]) {
+  using R = float;
   using S = CoopSizes<C>;
   constexpr int NT = S::NT, NK = (NT + 31) / 32;
   R* const stage = s + C::NSLOT;
@@ -774,7 +738,7 @@ __device__ __forceinline__ void coop_nodes(const PB* __restrict__ pbase, const K
       }
       const R T = a.p * rp * (PQ[0] * PQ[0] + PQ[1] * PQ[1] + PQ[2] * PQ[2]);
       R B[C::L + 1];
-      BoysSel<C::L, R>::eval(T, kc, B);
+      BoysFloat<C::L>::eval(T, kc, B);
       const R pref = a.K * c.K * rs;
 #pragma unroll
       for (int m = 0; m <= C::L; ++m) cv[HF_NCOEF + m] = B[m] * pref;
@@ -825,7 +789,7 @@ __device__ __forceinline__ void coop_block(const PairSet& P, const KernelCommon&
   (void)ND;
   [[maybe_unused]] R acc[NK];
   if constexpr (std::is_same<R, float>::value)
-    coop_nodes<C, R>(P.prim32, kc, bra, ket, q_lo, nq, s, G, lane, acc);
+    coop_nodes<C>(P.prim32, kc, bra, ket, q_lo, nq, s, G, lane, acc);
   else
     coop_herm<C, R>(P, kc, bra, ket, q_lo, nq, s, lane);  // leaves them at s
   // contracted [e0|f0] -> shared memory, then HRR
@@ -1038,7 +1002,7 @@ __global__ void __launch_bounds__(128) eri_schwarz_coop_kernel(const int* __rest
   if (lane == 0) Q[pid] = sqrt(m);
 }
 
-// Primitive quartets set up per pass: the class default, or HF_COOP_G
+// Primitive quartets an FP32 range sets up per pass: the class default, or HF_COOP_G
 // (8, 16 or 32) from the environment for tuning.
 template <class C>
 inline int coop_group() {
@@ -1155,8 +1119,9 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
 
 // Classes with L >= 5: one warp per quartet (part), the block from
 // coop_block.  What bounds it is what bounds the J/K kernel of the class
-// (FP64 issue).  A thread per quartet, the form before, kept the whole
-// [e0|f0] set of such a class in one thread and spilled it.
+// (the FP64 pipe).  A thread per quartet, the form before, kept the whole
+// [e0|f0] set of such a class in one thread and spilled it: the whole tensor of an
+// 11-atom s+p+d molecule took 985 ms, now 8.1 ms.
 template <class C>
 __global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
                                                              double* __restrict__ G, int nbf, const int g) {

@@ -25,8 +25,8 @@
 //    contributes below 2^-54 of the value to its error.  The table index and
 //    the offset come from the bits of y, without FP64 conversions.
 // (ps|ss), FP64: 0.0489 ns per primitive quartet on the whole GPU, from 0.0996
-// (the pipe's rate is 629e9 FP64 instructions x lanes per second: 31 of them,
-// from 63).
+// (the pipe's rate is 629e9 FP64 instructions x lanes per second: the time of
+// 31 of them, of which 27 are executed; 63 before).
 #pragma once
 #include <type_traits>
 #include <utility>
@@ -242,7 +242,7 @@ struct HPrim {
   R o2, P[3], PA[3], K;
 };
 __device__ __forceinline__ void load_hprim(const PairSet& s, int idx, HPrim<double>& q) {
-  const double* p = s.primh + (size_t)idx * PRIMH_STRIDE;
+  const double* p = s.prim64 + (size_t)idx * PRIM64_STRIDE;
   double v[8];
   asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
   asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v[4]), "=d"(v[5]), "=d"(v[6]), "=d"(v[7]) : "l"(p + 4));
@@ -250,7 +250,7 @@ __device__ __forceinline__ void load_hprim(const PairSet& s, int idx, HPrim<doub
   q.PA[0] = v[4]; q.PA[1] = v[5]; q.PA[2] = v[6]; q.K = v[7];
 }
 __device__ __forceinline__ void load_hprim(const PairSet& s, int idx, HPrim<df64>& q) {
-  const unsigned* p = reinterpret_cast<const unsigned*>(s.primhdf + (size_t)idx * 2 * PRIMH_STRIDE);
+  const unsigned* p = reinterpret_cast<const unsigned*>(s.primdf + (size_t)idx * PRIMDF_STRIDE);
   unsigned v[16];
   ldg256u(p, v);
   ldg256u(p + 8, v + 8);

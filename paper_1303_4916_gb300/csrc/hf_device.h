@@ -54,20 +54,19 @@ __host__ __device__ constexpr size_t boysydf_off(int L) {
 // generic cooperative kernel
 #define HF_DF_LMAX 4
 
-// Primitive-pair record, FP64: p, 1/(2p), P[3], PA[3], K, a (80 bytes; a
-// is the exponent of A's primitive, b = p - a); FP32: the same ten values
-// then two pads (48 bytes); df64: the ten values as (hi, lo) float pairs
-// (80 bytes).
+// Primitive-pair record, FP64: 1/(2p), P[3], PA[3], K'', p, K, a, one pad
+// (96 bytes; a is the exponent of A's primitive, b = p - a).  The Hermite
+// kernels read the first eight, two 32-byte loads, and as (hi, lo) float pairs
+// in df64 (64 bytes); the Rys kernels all but K''.  FP32: p, 1/(2p), P[3],
+// PA[3], K, a, two pads (48 bytes; the reduced-precision ranges).
 // K = c_a c_b exp(-ab/p |AB|^2) sqrt(2) pi^(5/4) / p, so that the
 // primitive-quartet prefactor 2 pi^(5/2) / (p q sqrt(p+q)) K_ab K_cd of
 // [00|00]^(m) is K_ab' K_cd' / sqrt(p+q).
-#define PRIM64_STRIDE 10
+// K'' = K 2^(1/4) (2p)^(-1/2): with s = 1/(2p) + 1/(2q) the prefactor
+// K_ab K_cd / sqrt(p+q) is K''_ab K''_cd / sqrt(s).
+#define PRIM64_STRIDE 12
 #define PRIM32_STRIDE 12
-#define PRIMDF_STRIDE 20
-// Record of the Hermite kernels: 1/(2p), P[3], PA[3], K'' = K 2^(1/4) (2p)^(-1/2)
-// (64 bytes; as (hi, lo) float pairs in df64).  With s = 1/(2p) + 1/(2q) the
-// prefactor K_ab K_cd / sqrt(p+q) is K''_ab K''_cd / sqrt(s).
-#define PRIMH_STRIDE 8
+#define PRIMDF_STRIDE 16
 
 // Shell pair (A, B) with l_A >= l_B: first basis functions of A and B,
 // offset and count of its significant primitive pairs (sorted by
@@ -82,11 +81,9 @@ struct PairSet {
   const double* prim64;
   const float* prim32;
   const PairInfo* info;
-  const float* primdf;
   int npairs;      // shell pairs (records of info)
   int nprimpairs;  // primitive-pair records
-  const double* primh;   // Hermite-kernel records, same order as prim64
-  const float* primhdf;
+  const float* primdf;   // the (hi, lo) records, same order as prim64
 };
 
 #define HF_NPAIRCLASS 15  // (la, lb), la >= lb, l <= 4

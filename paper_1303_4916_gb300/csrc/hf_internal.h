@@ -145,8 +145,6 @@ struct hf_basis {
   DevArray<double> prim64;
   DevArray<float> prim32;
   DevArray<float> primdf;
-  DevArray<double> primh;             // records of the Hermite kernels, FP64 and (hi, lo) floats
-  DevArray<float> primhdf;
   DevArray<PairInfo> pinfo;
   DevArray<double> Q;                 // per pair
   std::vector<double> Q_h;
@@ -192,8 +190,7 @@ struct hf_basis {
 int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned flags);
 
 inline PairSet hf_pairset(const hf_basis* b) {
-  return PairSet{b->prim64.ptr, b->prim32.ptr, b->pinfo.ptr, b->primdf.ptr, b->npairs, b->nprimpairs, b->primh.ptr,
-                 b->primhdf.ptr};
+  return PairSet{b->prim64.ptr, b->prim32.ptr, b->pinfo.ptr, b->npairs, b->nprimpairs, b->primdf.ptr};
 }
 // Boys function of the reduced-precision (FP32) quartets: FP32 with
 // HF_JK_FP32_BOYS; else df64 in the df64 tier (the tier's stand-in for FP64);

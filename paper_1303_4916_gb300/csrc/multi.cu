@@ -160,7 +160,7 @@ int MultiJK::launch(const KernelCommon& kc, double* class_ms) {
   const dim3 g(std::max(1, 2 * ctx->num_sms / std::max(1, nmol)), nmol);
   zero_jk_batch<<<g, 256, 0, st>>>(table.ptr);
   HF_CUDA(cudaMemsetAsync(counters.ptr, 0, sizeof(int) * 2 * HF_NCLASS, st));
-  const PairSet none{nullptr, nullptr, nullptr, nullptr};
+  const PairSet none{};
   const MolJK one{};
   cudaEvent_t ev[2] = {nullptr, nullptr};
   if (class_ms) {

@@ -27,6 +27,11 @@
 // in registers; the finished chunk is digested into J and K as the
 // cooperative kernels do (same symmetry weights and accumulators).  The
 // smallest f/g classes run one quartet per lane instead (rys_thread.cu).
+// FP64 instructions bound it, so the binomials and component scales of a quartet's
+// set-up come from constant tables, and a block just above one chunk is cut evenly
+// (the 60 rows of (fd|dp) went as 56 and 4, at full cost each): a build of
+// QZ-shaped water (140 functions, s to g) 21.4 -> 16.2 ms with both.  Finer items
+// (24 to 8 steps instead of 16 primitive quartets) gained nothing.
 // The gradient's derivative kernel (rys_grad.cu) builds the same tables,
 // one power higher on A, B and C.
 #include <algorithm>
@@ -367,17 +372,17 @@ __device__ void rys_rows(const RysClass& rc, const double* __restrict__ prim, co
     const int ib = qq / nk, ik = qq - ib * nk;
     const double* rb = prim + (size_t)(bra.prim0 + ib) * PRIM64_STRIDE;
     const double* rk = prim + (size_t)(ket.prim0 + ik) * PRIM64_STRIDE;
-    const double p = __ldg(rb), q = __ldg(rk);
-    const double PQx = __ldg(rb + 2) - __ldg(rk + 2), PQy = __ldg(rb + 3) - __ldg(rk + 3),
-                 PQz = __ldg(rb + 4) - __ldg(rk + 4);
+    const double p = __ldg(rb + 8), q = __ldg(rk + 8);
+    const double PQx = __ldg(rb + 1) - __ldg(rk + 1), PQy = __ldg(rb + 2) - __ldg(rk + 2),
+                 PQz = __ldg(rb + 3) - __ldg(rk + 3);
     const double ipq = 1.0 / (p + q);
     const double T = p * q * ipq * (PQx * PQx + PQy * PQy + PQz * PQz);
-    const double pref = __ldg(rb + 8) * __ldg(rk + 8) * sqrt(ipq);
+    const double pref = __ldg(rb + 9) * __ldg(rk + 9) * sqrt(ipq);
     if (lane < rc.n) rys_rule_root(rtab, rc.n, lane, T, ru + lane, rw + lane);
     const double qf = q * ipq, pf = p * ipq;
     const double PQg = gdir == 0 ? PQx : (gdir == 1 ? PQy : PQz);
-    const double PAg = __ldg(rb + 5 + gdir), QCg = __ldg(rk + 5 + gdir);
-    const double hp = __ldg(rb + 1), hq = __ldg(rk + 1);  // 1/(2p), 1/(2q)
+    const double PAg = __ldg(rb + 4 + gdir), QCg = __ldg(rk + 4 + gdir);
+    const double hp = __ldg(rb), hq = __ldg(rk);  // 1/(2p), 1/(2q)
     __syncwarp();
     for (int r = 0; r < rc.n; ++r) {
       const double u = ru[r];

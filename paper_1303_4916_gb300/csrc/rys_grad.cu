@@ -270,21 +270,21 @@ __global__ void __launch_bounds__(128) rys_grad_kernel(const JKWork w, const Pai
           const int ibp = qq / nk, ikp = qq - ibp * nk;
           const double* rb = ps.prim64 + (size_t)(bra.prim0 + ibp) * PRIM64_STRIDE;
           const double* rk = ps.prim64 + (size_t)(ket.prim0 + ikp) * PRIM64_STRIDE;
-          const double p = __ldg(rb), q = __ldg(rk), s = p + q;
-          const double PQ[3] = {__ldg(rb + 2) - __ldg(rk + 2), __ldg(rb + 3) - __ldg(rk + 3),
-                                __ldg(rb + 4) - __ldg(rk + 4)};
+          const double p = __ldg(rb + 8), q = __ldg(rk + 8), s = p + q;
+          const double PQ[3] = {__ldg(rb + 1) - __ldg(rk + 1), __ldg(rb + 2) - __ldg(rk + 2),
+                                __ldg(rb + 3) - __ldg(rk + 3)};
           const double rs = hfk::hf_rsqrt(s);
           double ipq = rs * rs;
           ipq = fma(ipq, fma(-s, ipq, 1.0), ipq);
           const double qf = q * ipq, pf = p * ipq;
           double u, wt;
           rys_rule_root(kc.rys, gc.n, root, p * qf * fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], PQ[2] * PQ[2])), &u, &wt);
-          const double g0z = live ? wt * (__ldg(rb + 8) * __ldg(rk + 8) * rs) : 0.0;
-          const double B00 = 0.5 * u * ipq, B10 = __ldg(rb + 1) * (1.0 - u * qf), B01 = __ldg(rk + 1) * (1.0 - u * pf);
+          const double g0z = live ? wt * (__ldg(rb + 9) * __ldg(rk + 9) * rs) : 0.0;
+          const double B00 = 0.5 * u * ipq, B10 = __ldg(rb) * (1.0 - u * qf), B01 = __ldg(rk) * (1.0 - u * pf);
           const double uq = u * qf, up = u * pf;
           if (wide) {  // G(gn, 0 .. MG) of direction gdir on this lane, G(gn - 1, m) from the lane below
             const double PQg = gdir == 0 ? PQ[0] : (gdir == 1 ? PQ[1] : PQ[2]);
-            const double c00 = __ldg(rb + 5 + gdir) - uq * PQg, d00 = __ldg(rk + 5 + gdir) + up * PQg;
+            const double c00 = __ldg(rb + 4 + gdir) - uq * PQg, d00 = __ldg(rk + 4 + gdir) + up * PQg;
             double gg = gdir == 2 ? g0z : 1.0, gp = 0.0;
             for (int k = 0; k < gn; ++k) {
               const double tt = fma(c00, gg, kBin.k[k] * B10 * gp);
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128) rys_grad_kernel(const JKWork w, const Pai
           } else {  // one lane per direction, or one lane for all
             for (int dir = sub; dir < 3; dir += gc.g) {
               const double PQg = dir == 0 ? PQ[0] : (dir == 1 ? PQ[1] : PQ[2]);
-              const double c00 = __ldg(rb + 5 + dir) - uq * PQg, d00 = __ldg(rk + 5 + dir) + up * PQg;
+              const double c00 = __ldg(rb + 4 + dir) - uq * PQg, d00 = __ldg(rk + 4 + dir) + up * PQg;
               double* const Gd = tb + dir * gc.SG;
               double gg = dir == 2 ? g0z : 1.0, gp = 0.0;
               Gd[0] = gg;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(128) rys_grad_kernel(const JKWork w, const Pai
             }
             __syncwarp();
           }
-          const double za2 = 2.0 * __ldg(rb + 9), zb2 = 2.0 * (p - __ldg(rb + 9)), zc2 = 2.0 * __ldg(rk + 9);
+          const double za2 = 2.0 * __ldg(rb + 10), zb2 = 2.0 * (p - __ldg(rb + 10)), zc2 = 2.0 * __ldg(rk + 10);
 #pragma unroll
           for (int dir = 0; dir < 3; ++dir) {
             const double* const X = tb + gc.oI + dir * gc.SI;
