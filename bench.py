@@ -130,31 +130,31 @@ DF_ADD, DF_MUL, DF_FMA, DF_RSQRT = 11, 7, 15, 25
 
 def df64_ops_per_prim_quartet(la, lb, lc, ld, vrr_flops):
     """FP32 operations per primitive quartet of the df64 thread-per-quartet
-    kernel of class (la lb|lc ld): set-up (p+q, 1/sqrt, 1/(p+q), rho/zeta and
-    rho/eta where used, PQ, WP and WQ where used, T, prefactor, scaling of the
-    L+1 B_m), the df64 Boys evaluation (row index and x 13; Horner of F_L 79;
-    for L >= 1 the exp series 79, its product 7, 2T 2 and L downward steps of
-    25) and the VRR, whose generated multiply-adds run as fused df64 steps
-    (15 FP32 operations per two counted flops)."""
+    kernel of class (la lb|lc ld), counted in herm.cuh: set-up (1/(2p) +
+    1/(2q), 1/sqrt and its square, rho/zeta and rho/eta, PQ, WP and WQ where
+    used, |PQ|^2 and y, prefactor, scaling of the L+1 B_m), the tabulated S_m
+    (offset 12; one row of 31 for L = 0, else z/3 7 and 45 per order) and the
+    VRR, whose generated multiply-adds run as fused df64 steps (15 FP32
+    operations per two counted flops)."""
     L = la + lb + lc + ld
     bra, ket = la + lb > 0, lc + ld > 0
-    setup = (DF_ADD                    # p + q
-             + DF_RSQRT + DF_MUL       # (p+q)^-1/2 and its square
-             + DF_MUL + DF_MUL * ket   # rho/zeta (T needs it), rho/eta
+    setup = (DF_ADD                    # 1/(2p) + 1/(2q)
+             + DF_RSQRT + DF_MUL       # its ^-1/2 and the square
+             + DF_MUL * bra + DF_MUL * ket   # rho/zeta, rho/eta
              + 3 * DF_ADD              # PQ
              + 3 * DF_MUL * bra + 3 * DF_MUL * ket   # WP, WQ
-             + 5 * DF_MUL + 2 * DF_ADD   # T = zeta (rho/zeta) |PQ|^2
+             + 2 * DF_MUL + 2 * DF_FMA  # y = w |PQ|^2
              + 2 * DF_MUL              # prefactor
-             + DF_MUL * (L + 1))       # B_m = prefactor F_m
-    boys = 13 + 79 + ((79 + DF_MUL + 2 + 25 * L) if L >= 1 else 0)
+             + DF_MUL * (L + 1))       # B_m = prefactor S_m
+    boys = 12 + (31 if L == 0 else DF_MUL + 45 * (L + 1))
     return setup + boys + vrr_flops * DF_FMA / 2.0
 
 
 def kernel_hash():
     """Hash of the source the dominant kernel, eri_jk_kernel<C_ps_ss, double>,
     is compiled from, with // comments removed: eri.cuh without the
-    cooperative (L >= 5) kernel's section and the launcher macros, the
-    generated C_ps_ss class and hf_device.h."""
+    cooperative (L >= 5) kernel's section and the launcher macros, herm.cuh,
+    the generated C_ps_ss class and hf_device.h."""
     import re
     csrc = os.path.join(ROOT, "paper_1303_4916_gb300", "csrc")
 
@@ -172,6 +172,10 @@ def kernel_hash():
     i = gen.find("struct C_ps_ss {")
     with open(os.path.join(csrc, "hf_device.h")) as fh:
         dev = fh.read()
+    herm = os.path.join(csrc, "herm.cuh")
+    if os.path.exists(herm):
+        with open(herm) as fh:
+            dev += fh.read()
     h = hashlib.sha256()
     for t in (part, gen[i:gen.find("\n};\n", i)], dev):
         h.update(code(t).encode())
@@ -572,6 +576,9 @@ def run_ours(args):
                      "kernel": f"eri_jk_kernel {cls_name} fp64",
                      "kernel_ms": dom_ms, "kernel_flops": flops[dom],
                      "peak_note": "FP64 CUDA-core nominal: 152 SM x 2 DFMA/clk x 2.07 GHz",
+                     "work_note": "flops are the Obara-Saika count of the unit of work, the same for every form; the "
+                                  "Hermite kernel needs fewer FP64 instructions for it and evaluates F_m's tail on "
+                                  "the FP32 pipe, so frac is work done against the FP64 peak and may pass 1",
                      "all_classes_tflops": all_flops / (all_ms * 1e-3) / 1e12},
         "roofline_df64": roofline_df64,
         "precision_modes": modes,
