@@ -2,6 +2,7 @@
 // quartet bucketing, the J/K launch sequence, one-electron integrals and the
 // stored-tensor path.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <numeric>
@@ -507,6 +508,11 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
   if (b->have_work && b->work_tau == tau && b->work_fp32 == fp32_bound && b->work_rys == rys) return HF_OK;
   hf_ctx* ctx = b->ctx;
   cudaStream_t st = ctx->stream;
+  struct Place {
+    double q;
+    int rank;
+  };
+  std::vector<Place> pos;
   for (int X = 0; X < HF_NPAIRCLASS; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       const int cls = X * (X + 1) / 2 + Y;
@@ -530,8 +536,17 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
         // positions of whole pairs in the unit list
         const int shift = chunk == 32 && r == 1 ? b->ketw_begin + yb - ub : 0;
         std::vector<int> bucket_prims(bk.empty() ? 0 : bk.size() - 1, 0);
+        // Schwarz factor and place by Q of each position, side by side for the
+        // searches (through the lists, three reads apart, the first build of
+        // a chain of 64 hydrogens took longer than before the units)
+        pos.resize(bk.empty() ? 0 : bk.back());
         for (size_t u = 0; u + 1 < bk.size(); ++u)
-          for (int k = bk[u]; k < bk[u + 1]; ++k) bucket_prims[u] = std::max(bucket_prims[u], prims_at(k));
+          for (int k = bk[u]; k < bk[u + 1]; ++k) {
+            const int pk = pair_at(k);
+            bucket_prims[u] = std::max(bucket_prims[u], prims_at(k));
+            pos[k] = {b->Q_h[pk], b->qrank[pk]};
+          }
+        const bool by_rank = X == Y && r == 0;
         for (int i = xb; i < xe; ++i) {
           const int pi = b->ketlist_h[i];
           const double qi = b->Q_h[pi];
@@ -545,9 +560,9 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
               }
               return lo;
             };
-            auto count_ge = [&](double thr) { return prefix([&](int k) { return qi * b->Q_h[pair_at(k)] >= thr; }); };
+            const int ri = by_rank ? b->qrank[pi] : INT_MAX;
+            auto count_ge = [&](double thr) { return prefix([&](int k) { return qi * pos[k].q >= thr && pos[k].rank <= ri; }); };
             int n = count_ge(tau);
-            if (X == Y && r == 0) n = std::min(n, prefix([&](int k) { return b->qrank[pair_at(k)] <= b->qrank[pi]; }));
             if (X == Y && r == 1) n = std::min(n, std::max(b0, i - xb + 1));
             const int m = fp32_bound > 0.0 ? std::min(count_ge(fp32_bound), n) : n;
             const int lo = r == 0 ? b0 : m, hi = r == 0 ? m : n;
