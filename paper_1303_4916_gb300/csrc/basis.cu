@@ -552,20 +552,24 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
           const double qi = b->Q_h[pi];
           for (size_t u = 0; u + 1 < bk.size(); ++u) {
             const int b0 = bk[u], b1 = bk[u + 1];
-            auto prefix = [&](auto&& keep) {  // first position in [b0, b1) that is not kept
-              int lo = b0, hi = b1;
+            const int ri = by_rank ? b->qrank[pi] : INT_MAX;
+            auto count_ge = [&](double thr, int top) {  // first position in [b0, top) that is not kept
+              int lo = b0, hi = top;
               while (lo < hi) {
                 const int mid = (lo + hi) / 2;
-                if (keep(mid)) lo = mid + 1; else hi = mid;
+                if (qi * pos[mid].q >= thr && pos[mid].rank <= ri) lo = mid + 1; else hi = mid;
               }
               return lo;
             };
-            const int ri = by_rank ? b->qrank[pi] : INT_MAX;
-            auto count_ge = [&](double thr) { return prefix([&](int k) { return qi * pos[k].q >= thr && pos[k].rank <= ri; }); };
-            int n = count_ge(tau);
-            if (X == Y && r == 1) n = std::min(n, std::max(b0, i - xb + 1));
-            const int m = fp32_bound > 0.0 ? std::min(count_ge(fp32_bound), n) : n;
-            const int lo = r == 0 ? b0 : m, hi = r == 0 ? m : n;
+            int lo = b0, hi;
+            if (r == 0) {
+              hi = count_ge(fp32_bound > 0.0 ? std::max(tau, fp32_bound) : tau, b1);
+            } else {
+              const int top = X == Y ? std::min(b1, i - xb + 1) : b1;
+              if (top <= b0) break;
+              hi = count_ge(tau, top);
+              lo = count_ge(fp32_bound, hi);
+            }
             if (hi <= lo) continue;
             bra[r].push_back(pi);
             kb[r].push_back(lo + shift);
