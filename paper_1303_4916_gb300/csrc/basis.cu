@@ -68,13 +68,18 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
     }
     order[j + 1] = o;
   }
-  int nsig = 0;
+  int nsig = 0, emin = 0, emax = 0;
   const int base = poff[t];
   for (int s = 0; s < n; ++s) {
     const int k = order[s];
-    if (mag[k] >= eps) ++nsig;
     const double a = exps[sh_prim[A] + k / KB], b = exps[sh_prim[B] + k % KB];
     const double p = a + b;
+    if (mag[k] >= eps) {
+      const int e = ilogb(2.0 * p);
+      emin = nsig ? min(emin, e) : e;
+      emax = nsig ? max(emax, e) : e;
+      ++nsig;
+    }
     const double K = coefs[sh_prim[A] + k / KB] * coefs[sh_prim[B] + k % KB] * exp(-a * b / p * r2) * 1.4142135623730951 *
                      pow(kPi, 1.25) / p;
     const double Px = (a * Ax + b * Bx) / p, Py = (a * Ay + b * By) / p, Pz = (a * Az + b * Bz) / p;
@@ -100,7 +105,8 @@ __global__ void pair_kernel(int npairs, const int* __restrict__ pA, const int* _
   pi.nprim = nsig;
   pi.AB[0] = ABx; pi.AB[1] = ABy; pi.AB[2] = ABz;
   pi.same = (A == B);
-  pi.pad = 0;
+  pi.emin = (short)emin;
+  pi.emax = (short)emax;
   info[t] = pi;
 }
 

@@ -790,8 +790,10 @@ __device__ __forceinline__ void coop_block(const PairSet& P, const KernelCommon&
   [[maybe_unused]] R acc[NK];
   if constexpr (std::is_same<R, float>::value)
     coop_nodes<C>(P.prim32, kc, bra, ket, q_lo, nq, s, G, lane, acc);
-  else
-    coop_herm<C, R>(P, kc, bra, ket, q_lo, nq, s, lane);  // leaves them at s
+  else if (std::is_same<R, double>::value || plain_range(bra, ket))  // leaves them at s
+    coop_herm<C, R, false>(P, kc, bra, ket, q_lo, nq, s, lane);
+  else if constexpr (std::is_same<R, df64>::value)
+    coop_herm<C, R, true>(P, kc, bra, ket, q_lo, nq, s, lane);
   // contracted [e0|f0] -> shared memory, then HRR
   R* const A = s;
   R* const H = s + NT;

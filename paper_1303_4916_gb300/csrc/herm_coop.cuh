@@ -12,6 +12,18 @@
 // (a J/K build of a 9-atom s+p+d molecule 22.7 -> 20.2 ms in FP64, of a 20-atom
 // one in df64 with an FP32 split 45 -> 36.4 ms).
 // Index tables (coop_tab.cu) are kept with the context.
+//
+// Range in df64: the set-up forms w^m, m <= 8, w = 2 rho up to twice the smaller
+// exponent, and floats end at 2^127: plain d shells of exponent 2500 overflow
+// (and a NaN follows), diffuse ones of 1e-3 lose their low words.  So a
+// quartet whose exponents leave the range where that cannot happen is taken in
+// powers of two: lengths in units of 2^-a, 4^a near its largest w, so that the
+// expansion coefficients are of order one; and per primitive quartet with k,
+// 4^k near w in those units, R^(m)_N is formed times 2^(-k (N + 2m)), which the
+// recursion keeps (PQ times 2^k, w times 4^-k), and the finished R_N is put
+// back by 2^(k N).  Only exponents change, so nothing is rounded by it.  It is an
+// instantiation of its own (SCALED): woven into the plain one, where it does
+// nothing, it cost a 20-atom build 1.4 %.
 #pragma once
 #include "herm.cuh"
 
@@ -104,6 +116,14 @@ __device__ __forceinline__ R coef_of(uint32_t w, const R* er, R first) {
   if (w >> 16) v = v * er[w >> 16];
   return v;
 }
+// times a power of two
+__device__ __forceinline__ df64 times_pow2(df64 a, float s) { return df64(a.hi * s, a.lo * s); }
+// The plain range of a quartet (all bounds on the exponent e of 2p, 2^e <= 2p):
+// w < 2^10 and >= 2^-7, prefactors of pairs below 2^14 (g w^8 of two d pairs
+// there is below 1e33 and, at the diffuse end, above 1e-25).
+__device__ __forceinline__ bool plain_range(const PairInfo& bra, const PairInfo& ket) {
+  return min(bra.emax, ket.emax) <= 9 && max(bra.emax, ket.emax) <= 13 && min(bra.emin, ket.emin) >= -6;
+}
 __device__ __forceinline__ double one_of(double) { return 1.0; }
 __device__ __forceinline__ df64 one_of(df64) { return df64(1.0f, 0.0f); }
 
@@ -120,12 +140,12 @@ __device__ __forceinline__ void store_e(R X, R h, R* er, int d) {
 }
 
 // The [e0|f0] of (bra|ket) over the primitive quartets [q_lo, q_hi) (bra
-// primitive major) into s[oA ..].
-template <class C, typename R>
+// primitive major) into s[oA ..]; SCALED outside the plain range.
+template <class C, typename R, bool SCALED>
 __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& kc, const PairInfo& bra,
                                           const PairInfo& ket, int q_lo, int q_hi, R* const s, const int lane) {
   using T = CoopTab<C>;
-  constexpr int L = T::L, LK = T::LK, LB = T::LB, NF = C::NF, NB = 32 / T::KC;
+  constexpr int L = T::L, LK = T::LK, LB = T::LB, NF = C::NF;
   const R zero = zero_of(R{});
   for (int k = lane; k < T::NA; k += 32) s[T::oA + k] = zero;
   if (q_hi <= q_lo) {  // an empty part, or a pair without significant primitives
@@ -143,6 +163,11 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
     pl[k] = __ldg(tab + T::P0 + tl * T::NUW + k);
   }
   const int ib_lo = q_lo / nk, ib_hi = (q_hi - 1) / nk + 1;
+  // lengths in units of 2^-ua; the bound keeps 2^(7 ua) a float
+  [[maybe_unused]] const int ua = SCALED ? max(-18, min(18, min(bra.emax, ket.emax) >> 1)) : 0;
+  [[maybe_unused]] int kq = 0;  // k of the primitive quartet of this lane's set-up row
+  auto len = [&](R x) { if constexpr (SCALED) return times_pow2(x, pow2f(ua)); else return x; };       // a length
+  auto area = [&](R x) { if constexpr (SCALED) return times_pow2(x, pow2f(2 * ua)); else return x; };  // 1 / (2p)
   R H[NF], X[NF];
   // e rows of the ket primitives [kb, ke), at most KC
   auto ket_rows = [&](int kb, int ke) {
@@ -151,7 +176,7 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
       if (kb + k < ke) {
         HPrim<R> c;
         load_hprim(P, ket.prim0 + kb + k, c);
-        store_e<LK, -1>(d == 0 ? c.PA[0] : d == 1 ? c.PA[1] : c.PA[2], c.o2, s + T::oE + k * T::NEK, d);
+        store_e<LK, -1>(len(d == 0 ? c.PA[0] : d == 1 ? c.PA[1] : c.PA[2]), area(c.o2), s + T::oE + k * T::NEK, d);
       }
     }
   };
@@ -166,16 +191,22 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
     HPrim<R> a, c;
     load_hprim(P, bra.prim0 + ib, a);
     load_hprim(P, ket.prim0 + ik, c);
-    const R rs = hf_rsqrt(a.o2 + c.o2);
-    const R w = rs * rs;
+    const R rs = hf_rsqrt(area(a.o2 + c.o2));
+    R w = rs * rs;
     R PQ[3];
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-      PQ[x] = a.P[x] - c.P[x];
+      PQ[x] = len(a.P[x] - c.P[x]);
       row[x] = PQ[x];
     }
     R B[L + 1];
     boys_y<L>(w * fmah(PQ[0], PQ[0], fmah(PQ[1], PQ[1], PQ[2] * PQ[2])), kc, B);
+    if constexpr (SCALED) {
+      kq = ((__float_as_int(w.hi) >> 23) - 127) >> 1;
+      w = times_pow2(w, pow2f(-2 * kq));
+#pragma unroll
+      for (int x = 0; x < 3; ++x) row[x] = times_pow2(PQ[x], pow2f(kq));
+    }
     R g = c.K * rs;
 #pragma unroll
     for (int m = 0; m <= L; ++m) {
@@ -183,9 +214,10 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
       if (m < L) g = g * w;
     }
   };
-  // Hermite integrals of n quartets from their rows, level by level, the lanes
-  // over all their entries (one quartet alone fills a third of them)
-  auto integrals = [&](const R* rows, int n) {
+  // Hermite integrals of n quartets from their rows (row0 on), level by level,
+  // the lanes over all their entries (one quartet alone fills a third of them)
+  auto integrals = [&](int row0, int n) {
+    const R* const rows = s + T::oRow + row0 * T::ROW;
     R* prev = L % 2 == 0 ? s + T::oR : s + T::oS;
     R* next = L % 2 == 0 ? s + T::oS : s + T::oR;
     if (lane < n) prev[lane * T::NR] = rows[lane * T::ROW + 3 + L];
@@ -205,6 +237,19 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
       prev = next;
       next = t;
     });
+    if constexpr (SCALED) {
+      for (int x0 = 0; x0 < n * T::NR; x0 += 32) {
+        const int x = x0 + lane, j = min(x / T::NR, n - 1), i = x - j * T::NR;
+        const int k = __shfl_sync(0xffffffffu, kq, row0 + j);
+        if (x < n * T::NR) {
+          int N = 0;
+#pragma unroll
+          for (int l = 0; l < L; ++l) N += i >= nherm(l);
+          s[T::oR + x] = times_pow2(s[T::oR + x], pow2f(k * N));
+        }
+      }
+      __syncwarp();
+    }
   };
   // H and the left-over X of n quartets, coefficients from ck on.  Both passes
   // go through one copy of the unrolled sums (they change places in between):
@@ -242,7 +287,7 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
     HPrim<R> a;
     load_hprim(P, bra.prim0 + ib, a);
     __syncwarp();
-    if (lane < 3) store_e<LB, 1>(lane == 0 ? a.PA[0] : lane == 1 ? a.PA[1] : a.PA[2], a.o2, s + T::oE, lane);
+    if (lane < 3) store_e<LB, 1>(len(lane == 0 ? a.PA[0] : lane == 1 ? a.PA[1] : a.PA[2]), area(a.o2), s + T::oE, lane);
     R* const Hs = s + T::oR;  // the integrals are done with
     if (sm == 0)
 #pragma unroll
@@ -288,7 +333,7 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
         for (int g = 0; g < ng; ++g) {
           const int kb = kr + g * (kt - kr) / ng, ke = kr + (g + 1) * (kt - kr) / ng;
           ket_rows(kb, ke);
-          integrals(s + T::oRow + (kb - kr) * T::ROW, ke - kb);
+          integrals(kb - kr, ke - kb);
           ket_coefs(ke - kb);  // over the second integral buffer
           __syncwarp();
           add_terms(s + T::oCK, ke - kb);
@@ -315,13 +360,23 @@ __device__ __forceinline__ void coop_herm(const PairSet& P, const KernelCommon& 
           const int k0 = max(kb, q_lo - ib * nk), k1 = min(ke, q_hi - ib * nk), n = k1 - k0;
           if (n <= 0) continue;  // warp-uniform
           clear();
-          integrals(s + T::oRow + ((ib - ib0) * T::KC + k0 - kb) * T::ROW, n);
+          integrals((ib - ib0) * T::KC + k0 - kb, n);
           add_terms(s + T::oCK + (k0 - kb) * T::NCK, n);
           flush(ib, n);
         }
       }
     }
   }
+  if constexpr (SCALED)  // [e0|f0] have the dimension length^(e + f - 1)
+    for (int o = lane; o < T::NA; o += 32) {
+      const int e = set0(C::LA) + o / NF, f = set0(C::LC) + o % NF;
+      int l = 0;
+#pragma unroll
+      for (int i = 0; i < LB; ++i) l += e >= nherm(i);
+#pragma unroll
+      for (int i = 0; i < LK; ++i) l += f >= nherm(i);
+      s[T::oA + o] = times_pow2(s[T::oA + o], pow2f(ua * (1 - l)));
+    }
 }
 
 }  // namespace hfk

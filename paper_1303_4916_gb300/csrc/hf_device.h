@@ -70,11 +70,14 @@ __host__ __device__ constexpr size_t boysydf_off(int L) {
 
 // Shell pair (A, B) with l_A >= l_B: first basis functions of A and B,
 // offset and count of its significant primitive pairs (sorted by
-// magnitude), AB = A - B, same = (A == B).
+// magnitude), AB = A - B, same = (A == B), and the least and the largest
+// binary exponent of 2p among its significant primitive pairs (zeros when it
+// has none).
 struct PairInfo {
   int bfA, bfB, prim0, nprim;
   double AB[3];
-  int same, pad;
+  int same;
+  short emin, emax;
 };
 
 struct PairSet {
