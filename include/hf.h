@@ -276,8 +276,10 @@ int hf_fock_jk_noalloc(hf_basis* b, const double* D, double* J, double* K, const
 int hf_one_electron(hf_basis* b, double* S, double* T, double* V, double* e_nuc);
 
 /* Full ERI tensor G[i][j][k][l] = (ij|kl) of Eq. 5 into a DEVICE buffer of
- * nbf^4 doubles (nbf <= HF_STORED_NBF_MAX; the caller allocates it).
- * Errors: HF_ERR_INVALID. */
+ * nbf^4 doubles (nbf <= HF_STORED_NBF_MAX; the caller allocates it).  Every
+ * element is the same to the last bit on every call for the same basis, and on
+ * all eight index permutations.  Scratch: up to 256 MB, kept by the context.
+ * Errors: HF_ERR_INVALID, HF_ERR_OOM. */
 int hf_eri_tensor(hf_basis* b, double* G);
 
 /* J and K from a stored ERI tensor G (device, nbf^4): J = G vec(D),

@@ -22,7 +22,7 @@ LIB = os.path.join(HERE, "libhf.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # heaviest first, so the long compiles start early
 SOURCES = ["rys_thread.cu", "eri_d6.cu", "eri_d5.cu", "eri_d4.cu", "eri_d3.cu", "eri_d2.cu", "eri_d1.cu", "eri_sp.cu",
-           "rys.cu", "coop_tab.cu", "rys_grad.cu", "grad.cu", "api.cu", "basis.cu", "onee.cu", "eig.cu", "scf.cu", "batch.cu", "serve.cu", "noalloc.cu", "multi.cu",
+           "rys.cu", "coop_tab.cu", "rys_grad.cu", "grad.cu", "api.cu", "basis.cu", "tensor.cu", "onee.cu", "eig.cu", "scf.cu", "batch.cu", "serve.cu", "noalloc.cu", "multi.cu",
            "mp2.cu"]
 KERNEL_HEADERS = ["eri.cuh", "herm.cuh", "herm_coop.cuh", "eri_classes.cuh", "hf_device.h", "rys.cuh", "rys_class.cuh", "df64.cuh"]
 HEADERS = KERNEL_HEADERS + ["hf_internal.h", "scf_internal.h", "multi.h", "../../include/hf.h"]

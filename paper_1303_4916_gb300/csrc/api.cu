@@ -337,6 +337,7 @@ void hf_ctx_teardown(hf_ctx* c) {
   if (c->cooptab) hf_dev_free(c, c->cooptab, 0);
   if (c->rys) hf_dev_free(c, c->rys, 0);
   if (c->grad_tabs) hf_grad_tabs_free(c->grad_tabs);
+  if (c->slots) hf_dev_free(c, c->slots, c->nslots * sizeof(double));
   if (c->bounds) hf_dev_free(c, c->bounds, 0);
   if (c->stream) cudaStreamSynchronize(c->stream);
   for (int k = 0; k < hf_ctx::kSide; ++k) {

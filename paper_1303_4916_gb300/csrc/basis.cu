@@ -175,6 +175,28 @@ __global__ void finish_fixed(const unsigned long long* __restrict__ Jq, const un
 // sizes as give the least lane time, sum over buckets of ceil(n / 32) times
 // the largest size.  A cap of 12 costs a digestion per 12 primitives of a
 // long ket; lower ones (3, 5, 9) measured the same from 8 atoms (43 us) to 15.
+std::vector<int> hf_lane_time_cuts(const long long* count, int nsize) {
+  std::vector<long long> best(nsize + 1, -1);  // for the sizes below z
+  std::vector<int> cut(nsize + 1, 0), out;
+  best[0] = 0;
+  for (int z = 1; z <= nsize; ++z) {
+    long long n = 0;
+    int top = 0;
+    for (int a = z - 1; a >= 0; --a) {  // last bucket: sizes a .. z - 1
+      n += count[a];
+      if (count[a] > 0 && top == 0) top = std::max(1, a);
+      const long long t = best[a] + (n + 31) / 32 * top;
+      if (best[z] < 0 || t < best[z]) {
+        best[z] = t;
+        cut[z] = a;
+      }
+    }
+  }
+  for (int z = nsize; z > 0; z = cut[z]) out.push_back(z);
+  out.push_back(0);
+  return out;
+}
+
 static void build_ket_units(hf_basis* b, const std::vector<int>& by_q) {
   const int np = b->npairs;
   constexpr int cap = 12;
@@ -188,32 +210,14 @@ static void build_ket_units(hf_basis* b, const std::vector<int>& by_q) {
       const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
       for (int u = 0; u < nu; ++u) ++count[(u + 1) * n / nu - u * n / nu];
     }
-    // least lane time over the ways to cut sizes 0..12 into neighbouring
-    // buckets: best[z] for sizes below z
-    long long best[14];
-    int cut[14];
-    best[0] = 0;
-    for (int z = 1; z <= 13; ++z) {
-      best[z] = -1;
-      long long n = 0;
-      int top = 0;
-      for (int a = z - 1; a >= 0; --a) {  // last bucket: sizes a .. z - 1
-        n += count[a];
-        if (count[a] > 0 && top == 0) top = std::max(1, a);
-        const long long t = best[a] + (n + 31) / 32 * top;
-        if (best[z] < 0 || t < best[z]) {
-          best[z] = t;
-          cut[z] = a;
-        }
-      }
-    }
+    const std::vector<int> cut = hf_lane_time_cuts(count, 13);
     b->ubuckets[X].push_back(0);
-    for (int z = 13; z > 0; z = cut[z]) {
+    for (size_t c = 0; c + 1 < cut.size(); ++c) {
       for (int r = 0; r < s1 - s0; ++r) {
         const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
         for (int u = 0; u < nu; ++u) {
           const int k0 = u * n / nu, k1 = (u + 1) * n / nu;
-          if (k1 - k0 >= cut[z] && k1 - k0 < z) b->ketu_h.push_back(make_int2(by_q[s0 + r], k0 << 16 | (k1 - k0)));
+          if (k1 - k0 >= cut[c + 1] && k1 - k0 < cut[c]) b->ketu_h.push_back(make_int2(by_q[s0 + r], k0 << 16 | (k1 - k0)));
         }
       }
       const int end = (int)b->ketu_h.size() - b->ketu_begin[X];
@@ -480,7 +484,7 @@ extern "C" int hf_basis_nshell(const hf_basis* b) { return b ? b->nshell : 0; }
 extern "C" size_t hf_basis_device_bytes(const hf_basis* b) {
   if (!b) return 0;
   size_t s = b->prim64.bytes() + b->prim32.bytes() + b->primdf.bytes() + b->ketu.bytes() + b->pinfo.bytes() + b->Q.bytes() + b->ketlist.bytes() +
-             b->counters.bytes() + b->hD.bytes() + b->hJ.bytes() + b->hK.bytes() + b->Dsum.bytes() + b->detq.bytes() + b->bfshell.bytes() + b->pairkey.bytes() + b->S.bytes() + b->T.bytes() +
+             b->counters.bytes() + b->hD.bytes() + b->hJ.bytes() + b->hK.bytes() + b->Dsum.bytes() + b->detq.bytes() + b->tensor.bytes() + b->S.bytes() + b->T.bytes() +
              b->V.bytes();
   for (int c = 0; c < HF_NCLASS; ++c)
     for (const ClassWork* w : {&b->work64[c], &b->work32[c]})
@@ -946,93 +950,6 @@ extern "C" int hf_fock_jk_uhf(hf_basis* b, const double* Da, const double* Db, d
   HF_CUDA(cudaGetLastError());
   HF_CHECK(hf_fock_jk_uhf_device(b, Da, Db, b->Dsum.ptr, J, Ka, Kb, o, nullptr));
   HF_CUDA(cudaStreamSynchronize(st));
-  return HF_OK;
-}
-
-// ------------------------------------------------------------- ERI tensor
-extern "C" int hf_eri_tensor(hf_basis* b, double* G) {
-  if (!b || !G) return hf_fail(HF_ERR_INVALID, "hf_eri_tensor: null argument");
-  if (b->nbf > HF_STORED_NBF_MAX)
-    return hf_fail(HF_ERR_INVALID, "hf_eri_tensor: nbf %d above %d", b->nbf, HF_STORED_NBF_MAX);
-  hf_ctx* ctx = b->ctx;
-  std::lock_guard<std::mutex> lk(ctx->mu);
-  cudaSetDevice(ctx->device);
-  HF_CHECK(hf_eri_tensor_device(b, G));
-  HF_CUDA(cudaStreamSynchronize(ctx->stream));
-  return HF_OK;
-}
-
-// The class kernels leave each unique quartet's block at (i j | k l) with i >=
-// j and k >= l in the order of its shell pairs and the bra pair's rank not
-// below the ket's; every other element is the copy of one of those.  One
-// block per row (i, j), a thread per (k, l), writes coalesced; the reads are
-// of the element's image, so HBM (one tensor read and written) bounds it.
-// key[A * ns + B] (pair of shells A, B in its own order) is the pair's rank
-// + 1, zero for the reversed order of two different shells.
-__global__ void mirror_tensor(double* __restrict__ G, int n, const int* __restrict__ bf_shell,
-                              const int* __restrict__ key, int ns) {
-  const int ij = blockIdx.x, i = ij / n, j = ij - i * n;
-  int kij = key[(size_t)bf_shell[i] * ns + bf_shell[j]];
-  const bool rij = kij == 0;
-  if (rij) kij = key[(size_t)bf_shell[j] * ns + bf_shell[i]];
-  const size_t nn = (size_t)n * n, bra = rij ? (size_t)j * n + i : (size_t)ij;
-  for (int kl = blockIdx.y * blockDim.x + threadIdx.x; kl < (int)nn; kl += gridDim.y * blockDim.x) {
-    const int k = kl / n, l = kl - k * n;
-    int kkl = key[(size_t)bf_shell[k] * ns + bf_shell[l]];
-    const bool rkl = kkl == 0;
-    if (rkl) kkl = key[(size_t)bf_shell[l] * ns + bf_shell[k]];
-    const size_t ket = rkl ? (size_t)l * n + k : (size_t)kl;
-    const bool sw = kij < kkl;
-    if (!(rij || rkl || sw)) continue;  // the element itself was written
-    G[(size_t)ij * nn + kl] = sw ? G[ket * nn + bra] : G[bra * nn + ket];
-  }
-}
-
-int hf_eri_tensor_device(hf_basis* b, double* G) {
-  hf_ctx* ctx = b->ctx;
-  cudaStream_t st = ctx->stream;
-  HF_CHECK(hf_basis_prepare_work(b, 0.0, 0.0, 0u));
-  const int n = b->nbf, ns = b->nshell;
-  const size_t nn = (size_t)n * n;
-  if (b->pairkey.n == 0) {
-    std::vector<int> key((size_t)ns * ns, 0), bfs(n);
-    for (int X = 0; X < HF_NPAIRCLASS; ++X)  // rank as in the work lists: by class, then by Q
-      for (int p = b->class_begin[X]; p < b->class_begin[X + 1]; ++p)
-        key[(size_t)b->pair_A[p] * ns + b->pair_B[p]] = b->class_begin[X] + b->qrank[p] + 1;
-    for (int s = 0; s < ns; ++s)
-      for (int k = b->sh_bf[s]; k < b->sh_bf[s + 1]; ++k) bfs[k] = s;
-    HF_CHECK(b->bfshell.alloc(ctx, n));
-    HF_CHECK(b->pairkey.alloc(ctx, key.size()));
-    const cudaError_t e1 = cudaMemcpyAsync(b->bfshell.ptr, bfs.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st);
-    const cudaError_t e2 =
-        cudaMemcpyAsync(b->pairkey.ptr, key.data(), sizeof(int) * key.size(), cudaMemcpyHostToDevice, st);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
-      b->pairkey.release();
-      return hf_fail(HF_ERR_CUDA, "tensor index upload: %s", cudaGetErrorString(cudaGetLastError()));
-    }
-  }
-  HF_CUDA(cudaMemsetAsync(G, 0, nn * nn * sizeof(double), st));
-  HF_CUDA(cudaMemsetAsync(b->counters.ptr, 0, sizeof(int) * 2 * HF_NCLASS, st));
-  const PairSet ps = hf_pairset(b);
-  const KernelCommon kc = hf_kernel_common(ctx, 0);
-  // heaviest classes first, forked onto the side streams as in hf_jk_run
-  HF_CUDA(cudaEventRecord(ctx->fork_ev, st));
-  for (int k = 0; k < hf_ctx::kSide; ++k) HF_CUDA(cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
-  int nside = 0;
-  for (int c = HF_NCLASS - 1; c >= 0; --c) {
-    ClassWork& w = b->work64[c];
-    if (w.w.nitems > 0)
-      ctx->ops[c].store(w.w, ps, kc, G, n, hf_launch_grid(ctx, 4, w.w.nitems), ctx->side[nside++ % hf_ctx::kSide]);
-  }
-  const cudaError_t launched = cudaGetLastError();
-  for (int k = 0; k < hf_ctx::kSide; ++k) {
-    HF_CUDA(cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
-    HF_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[k], 0));
-  }
-  HF_CUDA(launched);
-  const unsigned chunks = (unsigned)std::min<size_t>(std::max<size_t>(1, nn / 1024), 16);
-  mirror_tensor<<<dim3((unsigned)nn, chunks), 256, 0, st>>>(G, n, b->bfshell.ptr, b->pairkey.ptr, ns);
-  HF_CUDA(cudaGetLastError());
   return HF_OK;
 }
 

@@ -1060,20 +1060,14 @@ inline int coop_occupancy() {
 
 // ------------------------------------------------------------- ERI tensor kernels
 // The class kernels write each quartet's block once, at (i j | k l) with i,
-// j, k, l in the order of its shell pairs (bra pair first); mirror_tensor
-// (basis.cu) then copies it to the other index permutations.  An item that
-// is split along its primitive loop adds its part into the zeroed tensor.
-// Writing all eight images from here, as it was done before, cost up to
-// eight scattered 8-byte stores per integral and forbade the split, so that
-// a quartet of two 36-primitive pairs ran on one thread.
-__device__ __forceinline__ void store_eri(double* __restrict__ G, size_t idx, double v, bool add) {
-  if (add) atomicAdd(G + idx, v);
-  else G[idx] = v;
-}
-
+// j, k, l in the order of its shell pairs (bra pair first), or, where several
+// items share a quartet, each one's block in a slot of its own; tensor.cu adds the slots up in order and copies the blocks to the other index
+// permutations.  Writing all eight images from here cost up to eight scattered
+// 8-byte stores per integral and forbade the split, so that a quartet of two
+// 36-primitive pairs ran on one thread.
 template <class C>
 __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
-                                                        double* __restrict__ G, int nbf) {
+                                                        const StoreOut out) {
   constexpr int NA = C::NA, NB = C::NB, NC = C::NC, ND = C::ND;
   const int lane = threadIdx.x & 31;
   for (;;) {
@@ -1093,16 +1087,18 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
     const int kblk = rr / nsp, part = rr - kblk * nsp;
     const int kidx = __ldg(w.kbeg + bi) + 32 * kblk + lane;
     if (kidx >= __ldg(w.kend + bi)) continue;
-    const int2 unit = __ldg(w.ketu + kidx);
+    const int4 unit = __ldg(out.unit + kidx);
     const PairInfo bra = ps.info[bp];
     const PairInfo ket = ps.info[unit.x];
-    const bool add = nsp > 1 || (unit.y & 0xffff) < ket.nprim;
+    double* const mine = nsp == 1 && unit.w == 0
+                             ? nullptr
+                             : out.part + __ldg(out.slot + bi) + ((size_t)unit.z * nsp + part) * (NA * NB * NC * ND);
     const int ib0 = part * bra.nprim / nsp, ib1 = (part + 1) * bra.nprim / nsp;
     double acc[C::NE * C::NF];
     contracted<C, double>(ps, kc, bra.prim0 + ib0, ib1 - ib0, ket.prim0 + (unit.y >> 16), unit.y & 0xffff, acc);
     double I[NA * NB * NC * ND];
     C::template hrr<double>(acc, I, bra.AB, ket.AB);
-    const size_t n = (size_t)nbf;
+    const size_t n = (size_t)out.nbf;
 #pragma unroll
     for (int a = 0; a < NA; ++a)
 #pragma unroll
@@ -1111,10 +1107,11 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
         for (int c = 0; c < NC; ++c)
 #pragma unroll
           for (int d = 0; d < ND; ++d) {
-            const double v = I[((a * NB + b) * NC + c) * ND + d] * comp_scale(C::LA, a) * comp_scale(C::LB, b) *
+            const int o = ((a * NB + b) * NC + c) * ND + d;
+            const double v = I[o] * comp_scale(C::LA, a) * comp_scale(C::LB, b) *
                              comp_scale(C::LC, c) * comp_scale(C::LD, d);
             const size_t i = bra.bfA + a, j = bra.bfB + b, k = ket.bfA + c, l = ket.bfB + d;
-            store_eri(G, ((i * n + j) * n + k) * n + l, v, add);
+            (mine ? mine[o] : out.G[((i * n + j) * n + k) * n + l]) = v;
           }
   }
 }
@@ -1126,7 +1123,7 @@ __global__ void __launch_bounds__(128) eri_store_kernel(const JKWork w, const Pa
 // 11-atom s+p+d molecule took 985 ms, now 8.1 ms.
 template <class C>
 __global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
-                                                             double* __restrict__ G, int nbf, const int g) {
+                                                             const StoreOut out, const int g) {
   using S = CoopSizes<C>;
   constexpr int NB = C::NB, ND = C::ND, NF = C::NF, NAB = S::NAB, NCD = S::NCD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1153,25 +1150,27 @@ __global__ void __launch_bounds__(128) eri_store_coop_kernel(const JKWork w, con
     coop_block<C, double>(ps, kc, bra, ket, part * nq / nsp, (part + 1) * nq / nsp, s, g, lane);
     __syncwarp();
     const double* const Id = s + S::NT + NAB * NF;  // scaled by the d components
-    const size_t n = (size_t)nbf;
+    const long long slot = __ldg(out.slot + lo);
+    double* const mine = slot < 0 ? nullptr : out.part + slot + (size_t)(kj * nsp + part) * (NAB * NCD);
+    const size_t n = (size_t)out.nbf;
     for (int o = lane; o < NAB * NCD; o += 32) {
       const int ab = o / NCD, cd = o - ab * NCD;
       const size_t i = bra.bfA + ab / NB, j = bra.bfB + ab % NB, k = ket.bfA + cd / ND, l = ket.bfB + cd % ND;
-      store_eri(G, ((i * n + j) * n + k) * n + l, Id[o], nsp > 1);
+      (mine ? mine[o] : out.G[((i * n + j) * n + k) * n + l]) = Id[o];
     }
     __syncwarp();
   }
 }
 
 template <class C>
-inline void store_coop_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, double* G, int nbf, int grid,
+inline void store_coop_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const StoreOut& out, int grid,
                               cudaStream_t s) {
   const int g = coop_group<C>();
   const size_t sm = coop_smem_bytes<C, double>(g);
   static const cudaError_t attr =  // set once per process
       cudaFuncSetAttribute(eri_store_coop_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   (void)attr;
-  eri_store_coop_kernel<C><<<grid, 128, sm, s>>>(w, ps, kc, G, nbf, g);
+  eri_store_coop_kernel<C><<<grid, 128, sm, s>>>(w, ps, kc, out, g);
 }
 
 // ------------------------------------------------------------- Schwarz kernel
@@ -1264,12 +1263,12 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
     static const int n = occ_jkdf_query_##CLS();                                                         \
     return n;                                                                                            \
   }                                                                                                      \
-  static void launch_store_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc, double* G,   \
-                                 int nbf, int grid, cudaStream_t s) {                                    \
+  static void launch_store_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc,              \
+                                 const StoreOut& out, int grid, cudaStream_t s) {                        \
     if constexpr (hfgen::CLS::COOP)                                                                      \
-      hfk::store_coop_launch<hfgen::CLS>(w, ps, kc, G, nbf, grid, s);                                    \
+      hfk::store_coop_launch<hfgen::CLS>(w, ps, kc, out, grid, s);                                       \
     else                                                                                                 \
-      hfk::eri_store_kernel<hfgen::CLS><<<grid, 128, 0, s>>>(w, ps, kc, G, nbf);                         \
+      hfk::eri_store_kernel<hfgen::CLS><<<grid, 128, 0, s>>>(w, ps, kc, out);                            \
   }                                                                                                      \
   static void launch_schwarz_##CLS(const int* pairs, int npairs, const PairSet& ps, const KernelCommon& kc, \
                                    double* Q, cudaStream_t s) {                                          \

@@ -191,7 +191,20 @@ __host__ __device__ inline int class_index(int la, int lb, int lc, int ld) {
 // one warp per block when a class has few work items) on a stream.
 typedef void (*jk_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&, const MolJK&, const MolJK*, int grid,
                              int threads, cudaStream_t);
-typedef void (*store_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&, double*, int, int, cudaStream_t);
+// Where a tensor kernel leaves a block: at its place in the tensor G (nbf^4),
+// or, for a quartet that several items share, each one's block in its slot,
+// from part + slot[e] on.  Lists of one ket an item: by ket of the entry and
+// then part, where slot[e] >= 0.  Lists of 32: their ket units are here (.x the
+// pair, .y first << 16 | count, .z running number, .w the ket has several),
+// the slots by unit number and then part.
+struct StoreOut {
+  double* G;
+  double* part;
+  const long long* slot;  // [nbra]
+  const int4* unit;
+  int nbf;
+};
+typedef void (*store_launch_fn)(const JKWork&, const PairSet&, const KernelCommon&, const StoreOut&, int grid, cudaStream_t);
 typedef void (*schwarz_launch_fn)(const int*, int, const PairSet&, const KernelCommon&, double*, cudaStream_t);
 typedef int (*occ_fn)();
 struct EriClassOps {

@@ -47,6 +47,8 @@ struct hf_ctx {
   uint32_t* cooptab = nullptr;  // index tables of herm_coop.cuh
   double* rys = nullptr;    // Rys roots and weights table (rys.cuh)
   HfGradTabs* grad_tabs = nullptr;  // gradient class tables built so far (rys_grad.cu)
+  double* slots = nullptr;  // scratch of the dense tensor (tensor.cu)
+  size_t nslots = 0;
   EriClassOps ops[HF_NCLASS] = {};
   static constexpr int kSide = 8;
   cudaStream_t side[kSide] = {};     // class launches fork onto these
@@ -130,6 +132,32 @@ struct ClassWork {
   long long nquartets = 0;
 };
 
+// Quartets of bra pair `bra` with the kets from place ket0 of the pair list on
+// that have slots: nsplit for each unit of a ket, from `slot` on in the scratch
+// by running unit number (ints[unit0 + ket], -1: one unit each); `first` counts
+// elements.  na .. nd: components.
+struct HfSlotEntry {
+  int bra, ket0, nsplit, unit0;
+  long long slot, first;
+  unsigned char na, nb, nc, nd;
+};
+// The dense tensor's work lists (tensor.cu).
+struct HfTensorPlan {
+  bool ready = false;
+  DevArray<int> ints;         // every int list, in one copy
+  DevArray<int4> units;
+  DevArray<long long> slots;
+  DevArray<HfSlotEntry> entries;
+  size_t scratch = 0;         // doubles of the slots
+  long long nelement = 0;     // elements with slots
+  int nentry = 0;
+  JKWork w[HF_NCLASS] = {};
+  const long long* slot[HF_NCLASS] = {};
+  const int4* unit[HF_NCLASS] = {};
+  const int *key = nullptr, *bf_shell = nullptr;
+  size_t bytes() const { return ints.bytes() + units.bytes() + slots.bytes() + entries.bytes(); }
+};
+
 struct hf_basis {
   hf_ctx* ctx = nullptr;
   int natom = 0, nshell = 0, nbf = 0, nprim = 0, nelec = 0, lmax = 0;
@@ -176,8 +204,7 @@ struct hf_basis {
   // two 64-bit words per element
   DevArray<unsigned long long> detq;
 
-  // tensor path (lazily): shell of each function, rank of each oriented shell pair
-  DevArray<int> bfshell, pairkey;
+  HfTensorPlan tensor;  // tensor path (lazily)
 
   // one-electron data (lazily)
   DevArray<double> S, T, V;
@@ -266,4 +293,8 @@ void hf_grad_tabs_free(HfGradTabs* t);
 std::vector<uint32_t> hf_coop_tables();
 void hf_boysy_fill(uint32_t* t64, uint32_t* tdf);  // the S_m(y) tables, boysy64_off(LMAX + 1) and boysydf_off(LMAX + 1) words
 int hf_eri_tensor_device(hf_basis* b, double* G);
+// Cuts sizes 0 .. nsize - 1 (count[z] kets of size z) into buckets of
+// neighbouring sizes with the least lane time, sum over buckets of ceil(n / 32)
+// times the largest size: the boundaries from nsize down to 0.
+std::vector<int> hf_lane_time_cuts(const long long* count, int nsize);
 int hf_jk_stored_device(hf_basis* b, const double* G, const double* D, double* J, double* K);

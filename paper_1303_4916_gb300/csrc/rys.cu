@@ -580,12 +580,11 @@ __global__ void __launch_bounds__(128) rys_jk_kernel(const JKWork w, const PairS
   }
 }
 
-// Dense tensor: each quartet's block at the index order of its pairs (added
-// where the item covers a part of the primitive loop; mirror_tensor in
-// basis.cu copies it to the other permutations).
+// Dense tensor: each quartet's block at the index order of its pairs, or a
+// part's in its slot (tensor.cu finishes both).
 template <int KM>
 __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const PairSet ps, const KernelCommon kc,
-                                                        double* __restrict__ G, int nbf, const RysClass rc) {
+                                                        const StoreOut out, const RysClass rc) {
   extern __shared__ __align__(16) double rsm[];
   double* const s = rsm + (threadIdx.x >> 5) * rc.ws;
   const int lane = threadIdx.x & 31;
@@ -599,14 +598,13 @@ __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const Pa
     rys_item(w, t, &it);
     const int bp = __ldg(w.bra + it.bi);
     const PairInfo bra = ps.info[bp];
-    const bool add = it.nsp > (w.nchunk > 0 ? w.nchunk : 1);
+    const long long slot = __ldg(out.slot + it.bi);
+    const int nrange = it.nsp / w.nchunk, range = it.part / w.nchunk;
     for (int kidx = it.k0; kidx < it.k1; ++kidx) {
-      // lists of ket units (the thread-per-quartet f/g classes): the quartet
-      // goes with its ket's first unit
-      const int2 unit = w.chunk == 32 ? __ldg(w.ketu + kidx) : make_int2(__ldg(w.ket + kidx), 0);
-      if ((unit.y >> 16) != 0) continue;
-      const int kp = unit.x;
-      const PairInfo ket = ps.info[kp];
+      const PairInfo ket = ps.info[__ldg(w.ket + kidx)];
+      double* const mine =
+          slot < 0 ? nullptr
+                   : out.part + slot + (size_t)((kidx - __ldg(w.kbeg + it.bi)) * nrange + range) * (rc.na * NB * NCD);
       int q_lo, q_hi, c_lo, c_hi;
       rys_part(rc, w, bra, ket, it.part, it.nsp, &q_lo, &q_hi, &c_lo, &c_hi);
       if (q_hi <= q_lo) continue;
@@ -615,13 +613,13 @@ __global__ void __launch_bounds__(128) rys_store_kernel(const JKWork w, const Pa
         const int r0 = ch * rc.rpc, r1 = min(r0 + rc.rpc, rc.na * NB);
         rys_rows<KM>(rc, ps.prim64, kc.rys, bra, ket, q_lo, q_hi, r0, r1, s, lane);
         const double* I = s + rc.oBlk;
-        const size_t n = (size_t)nbf;
+        const size_t n = (size_t)out.nbf;
         for (int e = lane; e < (r1 - r0) * NCD; e += 32) {
           const int rl = e / NCD, cd = e - rl * NCD;
           const int row = r0 + rl, a = row / NB, b = row - a * NB;
           const int c = cd / ND, d = cd - c * ND;
           const size_t i = bra.bfA + a, j = bra.bfB + b, k = ket.bfA + c, l = ket.bfB + d;
-          hfk::store_eri(G, ((i * n + j) * n + k) * n + l, I[e], add);
+          (mine ? mine[r0 * NCD + e] : out.G[((i * n + j) * n + k) * n + l]) = I[e];
         }
         __syncwarp();
       }
@@ -713,12 +711,12 @@ int jk_occ() {
 }
 
 template <int CLS>
-void store_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, double* G, int nbf, int grid,
+void store_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const StoreOut& out, int grid,
                   cudaStream_t st) {
   static const RysClass rc = rys_class_of(CLS);
 #define RYS_S(KM)          \
   set_smem_attr_km<KM>(); \
-  rys_store_kernel<KM><<<grid, 128, smem_of(rc, 4), st>>>(w, ps, kc, G, nbf, rc)
+  rys_store_kernel<KM><<<grid, 128, smem_of(rc, 4), st>>>(w, ps, kc, out, rc)
   RYS_KM_DISPATCH(rc, RYS_S)
 #undef RYS_S
 }
