@@ -24,7 +24,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["rys_thread.cu", "eri_d6.cu", "eri_d5.cu", "eri_d4.cu", "eri_d3.cu", "eri_d2.cu", "eri_d1.cu", "eri_sp.cu",
            "rys.cu", "coop_tab.cu", "rys_grad.cu", "grad.cu", "api.cu", "basis.cu", "tensor.cu", "onee.cu", "eig.cu", "scf.cu", "batch.cu", "serve.cu", "noalloc.cu", "multi.cu",
            "mp2.cu"]
-KERNEL_HEADERS = ["eri.cuh", "herm.cuh", "herm_coop.cuh", "eri_classes.cuh", "hf_device.h", "rys.cuh", "rys_class.cuh", "df64.cuh"]
+KERNEL_HEADERS = ["eri.cuh", "herm.cuh", "herm_coop.cuh", "eri_classes.cuh", "hf_device.h", "per_device.h", "rys.cuh", "rys_class.cuh", "df64.cuh"]
 HEADERS = KERNEL_HEADERS + ["hf_internal.h", "scf_internal.h", "multi.h", "../../include/hf.h"]
 LMAX = 2
 

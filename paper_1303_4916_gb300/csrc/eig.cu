@@ -27,6 +27,7 @@
 
 #include "herm.cuh"
 #include "hf_internal.h"
+#include "per_device.h"
 #include "scf_internal.h"
 
 namespace {
@@ -285,9 +286,9 @@ size_t eig_smem(int n) {
 }  // namespace
 
 int hf_eig_small(hf_ctx* ctx, const EigJob* jobs, int count) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(HF_EIG_NMAX));
-  (void)attr;
+  static PerDevice limit;
+  if (hf_smem_limit(limit, eig_kernel, eig_smem(HF_EIG_NMAX)) < 0)
+    return hf_fail(HF_ERR_CUDA, "eigensolver's shared memory: %s", cudaGetErrorString(cudaGetLastError()));
   for (int c0 = 0; c0 < count; c0 += HF_EIG_BATCH) {
     EigBatch b{};
     const int k = std::min(HF_EIG_BATCH, count - c0);

@@ -28,6 +28,7 @@
 #include "eri_classes.cuh"
 #include "herm_coop.cuh"
 #include "hf_device.h"
+#include "per_device.h"
 #include "rys.cuh"
 
 namespace hfk {
@@ -1021,16 +1022,19 @@ inline size_t coop_smem_bytes(int g) {
   return (size_t)4 * CoopSizes<C>::template words<R>(g) * sizeof(R);
 }
 
+// the J/K kernel's shared-memory limit, which its launch and its occupancy both need
+template <class C, typename R>
+inline void coop_limit(size_t sm) {
+  static PerDevice limit;
+  hf_smem_limit(limit, eri_jk_coop_kernel<C, R>, sm);
+}
+
 template <class C, typename R>
 inline void coop_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const MolJK& one,
                         const MolJK* mols, int grid, int threads, cudaStream_t s) {
   const int g = coop_group<C>();
   const size_t sm = coop_smem_bytes<C, R>(g);
-  static bool attr = false;  // set once per process (same function on every device)
-  if (!attr) {
-    cudaFuncSetAttribute(eri_jk_coop_kernel<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  coop_limit<C, R>(sm);
   // shared memory per warp of the block (the attribute covers four warps)
   const size_t used = sm / 4 * (size_t)(threads / 32);
   eri_jk_coop_kernel<C, R><<<grid, threads, used, s>>>(w, ps, kc, one, mols, g);
@@ -1041,21 +1045,24 @@ inline void schwarz_coop_launch(const int* pairs, int npairs, const PairSet& ps,
                                 cudaStream_t s) {
   const int g = coop_group<C>();
   const size_t sm = coop_smem_bytes<C, double>(g);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(eri_schwarz_coop_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static PerDevice limit;
+  hf_smem_limit(limit, eri_schwarz_coop_kernel<C>, sm);
   eri_schwarz_coop_kernel<C><<<(npairs + 3) / 4, 128, sm, s>>>(pairs, npairs, ps, kc, Q, g);
 }
 
 template <class C, typename R>
 inline int coop_occupancy() {
   const size_t sm = coop_smem_bytes<C, R>(coop_group<C>());
-  cudaFuncSetAttribute(eri_jk_coop_kernel<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, eri_jk_coop_kernel<C, R>, 128, sm);
-  return n;
+  coop_limit<C, R>(sm);
+  static PerDevice blocks;
+  return hf_resident_blocks(blocks, eri_jk_coop_kernel<C, R>, 128, sm);
+}
+
+// the same of the thread-per-quartet kernel
+template <class C, typename R>
+inline int thread_occupancy() {
+  static PerDevice blocks;
+  return hf_resident_blocks(blocks, eri_jk_kernel<C, R>, 128, 0);
 }
 
 // ------------------------------------------------------------- ERI tensor kernels
@@ -1167,9 +1174,8 @@ inline void store_coop_launch(const JKWork& w, const PairSet& ps, const KernelCo
                               cudaStream_t s) {
   const int g = coop_group<C>();
   const size_t sm = coop_smem_bytes<C, double>(g);
-  static const cudaError_t attr =  // set once per process
-      cudaFuncSetAttribute(eri_store_coop_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  (void)attr;
+  static PerDevice limit;
+  hf_smem_limit(limit, eri_store_coop_kernel<C>, sm);
   eri_store_coop_kernel<C><<<grid, 128, sm, s>>>(w, ps, kc, out, g);
 }
 
@@ -1219,18 +1225,11 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
       hfk::eri_jk_kernel<hfgen::CLS, R><<<grid, threads, 0, s>>>(w, ps, kc, one, mols);                  \
   }                                                                                                      \
   template <typename R>                                                                                  \
-  static int occR_query_##CLS() {                                                                        \
-    int n = 0;                                                                                           \
+  static int occR_##CLS() {                                                                              \
     if constexpr (hfgen::CLS::COOP)                                                                      \
-      n = hfk::coop_occupancy<hfgen::CLS, R>();                                                          \
+      return hfk::coop_occupancy<hfgen::CLS, R>();                                                       \
     else                                                                                                 \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<hfgen::CLS, R>, 128, 0);      \
-    return n;                                                                                            \
-  }                                                                                                      \
-  template <typename R>                                                                                  \
-  static int occR_##CLS() { /* asked once: the same answer for every launch of the process */           \
-    static const int n = occR_query_##CLS<R>();                                                          \
-    return n;                                                                                            \
+      return hfk::thread_occupancy<hfgen::CLS, R>();                                                     \
   }                                                                                                      \
   static void launch_jk64_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const MolJK& one, \
                                 const MolJK* mols, int grid, int threads, cudaStream_t s) {              \
@@ -1249,19 +1248,11 @@ __global__ void __launch_bounds__(128) eri_schwarz_kernel(const int* __restrict_
     else                                                                                                 \
       launch_jkR_##CLS<double>(w, ps, kc, one, mols, grid, threads, s);                                  \
   }                                                                                                      \
-  static int occ_jkdf_query_##CLS() {                                                                    \
-    int n = 0;                                                                                           \
-    if constexpr (hfgen::CLS::COOP)                                                                      \
-      n = hfk::coop_occupancy<hfgen::CLS, df64>();                                                       \
-    else if constexpr (hfgen::CLS::L <= HF_DF_LMAX)                                                      \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<hfgen::CLS, df64>, 128, 0);   \
-    else                                                                                                 \
-      n = occR_##CLS<double>();                                                                          \
-    return n;                                                                                            \
-  }                                                                                                      \
   static int occ_jkdf_##CLS() {                                                                          \
-    static const int n = occ_jkdf_query_##CLS();                                                         \
-    return n;                                                                                            \
+    if constexpr (hfgen::CLS::COOP || hfgen::CLS::L <= HF_DF_LMAX)                                       \
+      return occR_##CLS<df64>();                                                                         \
+    else                                                                                                 \
+      return occR_##CLS<double>();                                                                       \
   }                                                                                                      \
   static void launch_store_##CLS(const JKWork& w, const PairSet& ps, const KernelCommon& kc,              \
                                  const StoreOut& out, int grid, cudaStream_t s) {                        \

@@ -44,6 +44,7 @@
 
 #include "eri.cuh"
 #include "hf_internal.h"
+#include "per_device.h"
 #include "rys.cuh"
 #include "rys_class.cuh"
 
@@ -662,13 +663,11 @@ size_t smem_of(const RysClass& rc, int warps) { return (size_t)warps * rc.ws * s
 
 template <int KM>
 void set_smem_attr_km() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    const int mx = 227 * 1024;
-    cudaFuncSetAttribute(rys_jk_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(rys_store_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(rys_schwarz_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  });
+  static PerDevice jk, store, schwarz;
+  const int mx = 227 * 1024;
+  hf_smem_limit(jk, rys_jk_kernel<KM>, mx);
+  hf_smem_limit(store, rys_store_kernel<KM>, mx);
+  hf_smem_limit(schwarz, rys_schwarz_kernel<KM>, mx);
 }
 
 // dispatch on the class's outputs per lane
@@ -697,17 +696,13 @@ void jk_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc, const
 
 template <int CLS>
 int jk_occ() {
-  static const int occ = [] {
-    const RysClass rc = rys_class_of(CLS);
-    int n = 0;
+  static const RysClass rc = rys_class_of(CLS);
+  static PerDevice blocks;
 #define RYS_O(KM)          \
   set_smem_attr_km<KM>(); \
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rys_jk_kernel<KM>, 128, smem_of(rc, 4))
-    RYS_KM_DISPATCH(rc, RYS_O)
+  return hf_resident_blocks(blocks, rys_jk_kernel<KM>, 128, smem_of(rc, 4))
+  RYS_KM_DISPATCH(rc, RYS_O)
 #undef RYS_O
-    return n;
-  }();
-  return occ;
 }
 
 template <int CLS>

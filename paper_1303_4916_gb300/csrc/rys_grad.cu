@@ -35,11 +35,11 @@
 #include <array>
 #include <cstring>
 #include <map>
-#include <mutex>
 #include <vector>
 
 #include "eri.cuh"
 #include "hf_internal.h"
+#include "per_device.h"
 #include "rys_class.cuh"
 
 namespace hfr {
@@ -428,10 +428,9 @@ int hf_grad_launch(hf_ctx* ctx, int cls, const JKWork& w, const PairSet& ps, con
       return hf_fail(HF_ERR_CUDA, "gradient table upload: %s", cudaGetErrorString(err));
     }
   }
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(rys_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  });
+  static PerDevice limit;
+  if (hf_smem_limit(limit, rys_grad_kernel, 227 * 1024) < 0)
+    return hf_fail(HF_ERR_CUDA, "gradient kernel's shared memory: %s", cudaGetErrorString(cudaGetLastError()));
   const size_t per_warp = (6 + (size_t)rc.rpc * rc.nc * rc.nd + 1 + (size_t)(32 / g) * e.gc.ws) * sizeof(double);
   int warps = 4;
   while (warps > 1 && warps * per_warp > 200 * 1024) warps /= 2;

@@ -49,13 +49,8 @@ void jk_thread_launch(const JKWork& w, const PairSet& ps, const KernelCommon& kc
 }
 template <int CLS>
 int jk_thread_occ() {
-  static const int occ = [] {  // asked once per process
-    int n = 0;
-    if constexpr (thread_class(CLS))
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hfk::eri_jk_kernel<RysTOf<CLS>, double>, 128, 0);
-    return n;
-  }();
-  return occ;
+  if constexpr (thread_class(CLS)) return hfk::thread_occupancy<RysTOf<CLS>, double>();
+  else return 0;
 }
 
 template <size_t... I>
