@@ -207,21 +207,33 @@ static void build_ket_units(hf_basis* b, const std::vector<int>& by_q) {
     b->ubuckets[X].clear();
     long long count[13] = {};
     for (int r = 0; r < s1 - s0; ++r) {
-      const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
-      for (int u = 0; u < nu; ++u) ++count[(u + 1) * n / nu - u * n / nu];
+      const int n = b->nprim_sig_h[by_q[s0 + r]], nu = n <= cap ? 1 : (n + cap - 1) / cap;
+      if (nu == 1) ++count[n];
+      else
+        for (int u = 0; u < nu; ++u) ++count[(u + 1) * n / nu - u * n / nu];
     }
     const std::vector<int> cut = hf_lane_time_cuts(count, 13);
+    // each unit straight to its bucket: where the bucket of a size has its next place
+    int bucket[13], next[14] = {};
+    for (int z = 0, c = (int)cut.size() - 2; z < 13; ++z) {
+      while (z >= cut[c]) --c;
+      bucket[z] = c;
+    }
+    for (int z = 0; z < 13; ++z) next[bucket[z] + 1] += (int)count[z];
     b->ubuckets[X].push_back(0);
     for (size_t c = 0; c + 1 < cut.size(); ++c) {
-      for (int r = 0; r < s1 - s0; ++r) {
-        const int n = b->nprim_sig_h[by_q[s0 + r]], nu = std::max(1, (n + cap - 1) / cap);
-        for (int u = 0; u < nu; ++u) {
-          const int k0 = u * n / nu, k1 = (u + 1) * n / nu;
-          if (k1 - k0 >= cut[c + 1] && k1 - k0 < cut[c]) b->ketu_h.push_back(make_int2(by_q[s0 + r], k0 << 16 | (k1 - k0)));
-        }
+      next[c + 1] += next[c];
+      if (next[c + 1] > next[c]) b->ubuckets[X].push_back(next[c + 1]);
+    }
+    b->ketu_h.resize(b->ketu_begin[X] + next[cut.size() - 1]);
+    int2* const out = b->ketu_h.data() + b->ketu_begin[X];
+    for (int r = 0; r < s1 - s0; ++r) {
+      const int n = b->nprim_sig_h[by_q[s0 + r]], nu = n <= cap ? 1 : (n + cap - 1) / cap;
+      for (int u = 0, k0 = 0; u < nu; ++u) {
+        const int k1 = nu == 1 ? n : (u + 1) * n / nu;
+        out[next[bucket[k1 - k0]]++] = make_int2(by_q[s0 + r], k0 << 16 | (k1 - k0));
+        k0 = k1;
       }
-      const int end = (int)b->ketu_h.size() - b->ketu_begin[X];
-      if (end > b->ubuckets[X].back()) b->ubuckets[X].push_back(end);
     }
   }
   // the pairs whole, in the order of the pair list: the FP32 ranges (an FP32
@@ -523,6 +535,7 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
     int rank;
   };
   std::vector<Place> pos;
+  std::vector<int> end_keep, end_64, end_rank;
   for (int X = 0; X < HF_NPAIRCLASS; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       const int cls = X * (X + 1) / 2 + Y;
@@ -546,9 +559,7 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
         // positions of whole pairs in the unit list
         const int shift = chunk == 32 && r == 1 ? b->ketw_begin + yb - ub : 0;
         std::vector<int> bucket_prims(bk.empty() ? 0 : bk.size() - 1, 0);
-        // Schwarz factor and place by Q of each position, side by side for the
-        // searches (through the lists, three reads apart, the first build of
-        // a chain of 64 hydrogens took longer than before the units)
+        // Schwarz factor and place by Q of each position, side by side
         pos.resize(bk.empty() ? 0 : bk.back());
         for (size_t u = 0; u + 1 < bk.size(); ++u)
           for (int k = bk[u]; k < bk[u + 1]; ++k) {
@@ -557,28 +568,39 @@ int hf_basis_prepare_work(hf_basis* b, double tau, double fp32_bound, unsigned f
             pos[k] = {b->Q_h[pk], b->qrank[pk]};
           }
         const bool by_rank = X == Y && r == 0;
+        const double keep = r == 0 && fp32_bound > 0.0 ? std::max(tau, fp32_bound) : tau;
+        // Where each bucket's kept prefix ends moves one way while the bras go
+        // down in Q (the rank's end the other way), so it is followed from bra
+        // to bra and starts over where they go up.
+        const size_t nbk = bk.empty() ? 0 : bk.size() - 1;
+        end_keep.assign(nbk, 0);
+        end_64.assign(nbk, 0);
+        end_rank.assign(nbk, 0);
+        int rlast = INT_MAX;
         for (int i = xb; i < xe; ++i) {
-          const int pi = b->ketlist_h[i];
+          const int pi = b->ketlist_h[i], ri = b->qrank[pi];
           const double qi = b->Q_h[pi];
-          for (size_t u = 0; u + 1 < bk.size(); ++u) {
+          if (ri < rlast)
+            for (size_t u = 0; u < nbk; ++u) {
+              end_keep[u] = end_64[u] = bk[u + 1];
+              end_rank[u] = bk[u];
+            }
+          rlast = ri;
+          for (size_t u = 0; u < nbk; ++u) {
             const int b0 = bk[u], b1 = bk[u + 1];
-            const int ri = by_rank ? b->qrank[pi] : INT_MAX;
-            auto count_ge = [&](double thr, int top) {  // first position in [b0, top) that is not kept
-              int lo = b0, hi = top;
-              while (lo < hi) {
-                const int mid = (lo + hi) / 2;
-                if (qi * pos[mid].q >= thr && pos[mid].rank <= ri) lo = mid + 1; else hi = mid;
-              }
-              return lo;
-            };
-            int lo = b0, hi;
-            if (r == 0) {
-              hi = count_ge(fp32_bound > 0.0 ? std::max(tau, fp32_bound) : tau, b1);
-            } else {
+            int &ek = end_keep[u], &e6 = end_64[u], &er = end_rank[u];
+            while (ek > b0 && !(qi * pos[ek - 1].q >= keep)) --ek;
+            int lo = b0, hi = ek;
+            if (by_rank) {
+              while (er < b1 && pos[er].rank <= ri) ++er;
+              hi = std::min(hi, er);
+            }
+            if (r == 1) {
               const int top = X == Y ? std::min(b1, i - xb + 1) : b1;
               if (top <= b0) break;
-              hi = count_ge(tau, top);
-              lo = count_ge(fp32_bound, hi);
+              hi = std::min(hi, top);
+              while (e6 > b0 && !(qi * pos[e6 - 1].q >= fp32_bound)) --e6;
+              lo = std::min(e6, hi);
             }
             if (hi <= lo) continue;
             bra[r].push_back(pi);
