@@ -9,7 +9,7 @@
 //         + sum over unique quartets Gamma d(ab|cd)/dR + dE_nuc/dR,
 // the W term coming from the orthonormality of the orbitals.  The two-
 // electron part runs on the Rys derivative kernel of every class
-// (rys.cu); the one-electron part here, one warp per ordered pair (i, j)
+// (rys_grad.cu); the one-electron part here, one warp per ordered pair (i, j)
 // of basis functions, takes the derivatives with respect to the centre A
 // of function i:
 //   d phi_a / dA_x = 2 alpha phi_(a + 1_x) - a_x phi_(a - 1_x)

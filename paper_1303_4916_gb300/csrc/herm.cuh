@@ -19,11 +19,16 @@
 //    in the records' prefactors.
 //  * 1/sqrt is the hardware estimate and one third-order correction, four
 //    FP64 instructions (hf_rsqrt).
-//  * S_m is a tabulated FP64 value plus a Taylor tail of at most 2^-7 of it,
-//    evaluated in double-float arithmetic (48 bits) on the FP32 pipe: two
-//    FP64 additions per order instead of an eight-term FP64 Horner.  The tail
-//    contributes below 2^-54 of the value to its error.  The table index and
-//    the offset come from the bits of y, without FP64 conversions.
+//  * S_m is a tabulated FP64 value plus a Taylor tail of at most 2^-7 of it
+//    (2^-5.9 in the far rows), evaluated in double-float arithmetic (48 bits) on
+//    the FP32 pipe: two FP64 additions per order instead of an eight-term FP64
+//    Horner.  The table index and the offset come from the bits of y, without
+//    FP64 conversions.  Against 40-digit values the worst relative error is
+//    1.9 x 2^-53 below T = 60 and, above it, 2.0 up to m = 6, 4.2 at m = 7 and
+//    6.9 at m = 8, where the first term left out of the tail shows.  (The FP64
+//    Horner with downward recursion: 1.8 to 10.8 below T = 60 from L = 0 to 8,
+//    and the upward recursion 2.4 to 28 above it.)  In df64, in units of 2^-48:
+//    at most 1.9 for all orders (before: 1.4 to 5 below T = 60, 4.5 to 45 above).
 // (ps|ss), FP64: 0.0489 ns per primitive quartet on the whole GPU, from 0.0996
 // (the pipe's rate is 629e9 FP64 instructions x lanes per second: the time of
 // 31 of them, of which 27 are executed; 63 before).
@@ -163,7 +168,9 @@ __device__ __forceinline__ void boys_y(double y, const KernelCommon& kc, double*
   const float zl = (float)(int)(yl & 0x1fffffffu) * 0x1p-58f;
   const df64 z = df_quick_two_sum(zh, zl), z3 = third(z);
   unsigned r[ROW];
-  const unsigned* const row = kc.boysy64 + boysy64_off(L) + (size_t)(far ? i + (BOYSY64_NNEAR - 256) : i) * ROW;
+  unsigned at = far ? i + (BOYSY64_NNEAR - 256) : i;
+  if (!HF_BCHECK(kc, at < BOYSY64_NNEAR + BOYSY_NFAR, HF_BC_BOYS, at)) at = 0;
+  const unsigned* const row = kc.boysy64 + boysy64_off(L) + (size_t)at * ROW;
 #pragma unroll
   for (int j = 0; j < ROW; j += 8) ldg256u(row + j, r + j);
   auto pr = [&](int j) { return df64(__uint_as_float(r[P0 + 2 * (j - 1)]), __uint_as_float(r[P0 + 2 * (j - 1) + 1])); };
@@ -202,7 +209,9 @@ __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) 
     const float xh = __fsub_rn(yh, (float)i * (far ? 1.0f / 32.0f : 1.0f / 64.0f));  // exact (Sterbenz)
     const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl);
     unsigned r[8];
-    ldg256u(kc.boysydf + (size_t)(far ? i + (BOYSYDF0_NNEAR - 1024) : i) * 8, r);
+    int at = far ? i + (BOYSYDF0_NNEAR - 1024) : i;
+    if (!HF_BCHECK(kc, at >= 0 && at < BOYSYDF0_NNEAR + BOYSYDF0_NFAR, HF_BC_BOYS, at)) at = 0;
+    ldg256u(kc.boysydf + (size_t)at * 8, r);
     auto w = [&](int j) { return __uint_as_float(r[j]); };
     const float g = __fmaf_rn(w(7), z.hi * 0.25f, w(6));
     df64 f = df_quick_two_sum(w(4), __fmaf_rn(g, z.hi * (1.0f / 3.0f), w(5)));
@@ -218,7 +227,9 @@ __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) 
   const float xh = __fsub_rn(yh, (float)i * 0.125f);  // exact (Sterbenz)
   const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl), z3 = third(z);
   unsigned r[ROW];
-  const unsigned* const row = kc.boysydf + boysydf_off(L) + (size_t)(far ? i + (BOYSYDF_NNEAR - 256) : i) * ROW;
+  int at = far ? i + (BOYSYDF_NNEAR - 256) : i;
+  if (!HF_BCHECK(kc, at >= 0 && at < BOYSYDF_NNEAR + BOYSY_NFAR, HF_BC_BOYS, at)) at = 0;
+  const unsigned* const row = kc.boysydf + boysydf_off(L) + (size_t)at * ROW;
 #pragma unroll
   for (int j = 0; j < ROW; j += 8) ldg256u(row + j, r + j);
   auto pr = [&](int j) { return df64(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])); };
@@ -319,9 +330,10 @@ __device__ __forceinline__ void herm_e(R X, R h, R (&e)[I + 1][I + 1]) {
 
 // acc[e * NF + f] += over bra records [b0, b0 + nb) and ket records [k0, k0 +
 // nk) (nk differs per lane; 0 for an inactive lane).
-template <class C, typename R>
+template <class C>
 __device__ __forceinline__ void contracted_herm(const PairSet& ps, const KernelCommon& kc, int b0, int nb, int k0,
-                                                int nk, R* acc) {
+                                                int nk, double* acc) {
+  using R = double;
   constexpr int LBR = C::LA + C::LB, LK = C::LC + C::LD, L = LBR + LK;
   constexpr int NT = nherm(LBR), NF = C::NF, NE = C::NE;
   const R zero = zero_of(R{});
@@ -456,9 +468,10 @@ __device__ __forceinline__ void contracted_os(const PairSet& ps, const KernelCom
   }
 }
 
-// Which form a class takes.  FP64 is bound by its FP64 instruction count: the
-// Hermite form has fewer in every class but (ds|pp), where its 90 Hermite sums
-// spill.  df64 is bound by FP32 issue and by L1 (a lane's own ket record per
+// Which form a class takes, as measured.  FP64 is bound by its FP64 instruction
+// count, of which the Hermite form has fewer; (ds|pp), with 10 Hermite indices
+// over 9 ket components, is the one class where the Obara-Saika form is faster
+// all the same ((pp|pp) has as many sums, spills 2 KB and still gains).  df64 is bound by FP32 issue and by L1 (a lane's own ket record per
 // primitive quartet, as the ket loop is the inner one): the Obara-Saika order,
 // with the ket record loaded once, is the faster.  Hermite against
 // Obara-Saika, ns per primitive quartet on the whole GPU (40-atom s+p and
@@ -472,7 +485,7 @@ template <class C, typename R>
 __device__ __forceinline__ void contracted(const PairSet& ps, const KernelCommon& kc, int b0, int nb, int k0, int nk,
                                            R* acc) {
   constexpr bool ds_pp = C::LA == 2 && C::LB == 0 && C::LC == 1 && C::LD == 1;
-  if constexpr (std::is_same<R, double>::value && !ds_pp) contracted_herm<C, R>(ps, kc, b0, nb, k0, nk, acc);
+  if constexpr (std::is_same<R, double>::value && !ds_pp) contracted_herm<C>(ps, kc, b0, nb, k0, nk, acc);
   else contracted_os<C, R>(ps, kc, b0, nb, k0, nk, acc);
 }
 

@@ -264,6 +264,24 @@ extern "C" int hf_rys_rule(int n, double T, double* u, double* w) {
 // ------------------------------------------------------------- device side
 namespace hfr {
 
+// Cartesian powers of component c of a shell of angular momentum l (l <= 5),
+// packed x | y << 4 | z << 8, at [l (l+1) (l+2) / 6 + c]; order as in the
+// basis: x power from l down, then y power from l - x down.
+struct CartTable {
+  unsigned short v[56];
+};
+constexpr CartTable make_cart() {
+  CartTable t{};
+  int k = 0;
+  for (int l = 0; l <= 5; ++l)
+    for (int x = l; x >= 0; --x)
+      for (int y = l - x; y >= 0; --y) t.v[k++] = (unsigned short)(x | (y << 4) | ((l - x - y) << 8));
+  return t;
+}
+static __constant__ CartTable kCart = make_cart();
+
+__device__ __forceinline__ int cart(int l, int c) { return kCart.v[l * (l + 1) * (l + 2) / 6 + c]; }
+
 // Fixed part of a warp's shared slice (doubles): transfer coefficients of
 // the bra [3][6][6] and the ket, roots, weights; kHead in all.
 constexpr int kCb = 0, kCd = 108, kRu = 216, kRw = 225;

@@ -1,6 +1,6 @@
 // rys_class.cuh -- what the Rys kernels of rys.cu and rys_grad.cu share: the
-// Cartesian powers, the shape of a class (roots, components, output chunks)
-// and the reading of a work item.
+// shape of a class (roots, components, output chunks) and the reading of a work
+// item.
 #pragma once
 #include <algorithm>
 
@@ -9,24 +9,6 @@
 #include "rys.cuh"
 
 namespace hfr {
-
-// Cartesian powers of component c of a shell of angular momentum l (l <= 5),
-// packed x | y << 4 | z << 8, at [l (l+1) (l+2) / 6 + c]; order as in the
-// basis: x power from l down, then y power from l - x down.
-struct CartTable {
-  unsigned short v[56];
-};
-constexpr CartTable make_cart() {
-  CartTable t{};
-  int k = 0;
-  for (int l = 0; l <= 5; ++l)
-    for (int x = l; x >= 0; --x)
-      for (int y = l - x; y >= 0; --y) t.v[k++] = (unsigned short)(x | (y << 4) | ((l - x - y) << 8));
-  return t;
-}
-static __constant__ CartTable kCart = make_cart();
-
-__device__ __forceinline__ int cart(int l, int c) { return kCart.v[l * (l + 1) * (l + 2) / 6 + c]; }
 
 // Binomials, small integers and the component scales s(l, c) = sqrt((2l-1)!! /
 // ((2x-1)!! (2y-1)!! (2z-1)!!)) of the axial-normalised basis.
