@@ -193,7 +193,8 @@ __device__ __forceinline__ void boys_y(double y, const KernelCommon& kc, double*
 
 // The same in double-float throughout, with rows y_i = i / 8 in both ranges
 // (|z| <= 2^-5, one more float term): a table a quarter of the FP64 one's
-// size, since here the row loads are a larger share of the time.
+// size, since here the row loads are a larger share of the time.  The far index
+// is bounded: centres far enough apart (1e16 bohr) overflow y.
 template <int L>
 __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) {
   const bool far = y.hi >= 120.0f;
@@ -209,7 +210,7 @@ __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) 
     const float xh = __fsub_rn(yh, (float)i * (far ? 1.0f / 32.0f : 1.0f / 64.0f));  // exact (Sterbenz)
     const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl);
     unsigned r[8];
-    int at = far ? i + (BOYSYDF0_NNEAR - 1024) : i;
+    int at = far ? min(i, 4096) + (BOYSYDF0_NNEAR - 1024) : i;
     if (!HF_BCHECK(kc, at >= 0 && at < BOYSYDF0_NNEAR + BOYSYDF0_NFAR, HF_BC_BOYS, at)) at = 0;
     ldg256u(kc.boysydf + (size_t)at * 8, r);
     auto w = [&](int j) { return __uint_as_float(r[j]); };
@@ -227,7 +228,7 @@ __device__ __forceinline__ void boys_y(df64 y, const KernelCommon& kc, df64* S) 
   const float xh = __fsub_rn(yh, (float)i * 0.125f);  // exact (Sterbenz)
   const df64 z = df_quick_two_sum(0.5f * xh, 0.5f * yl), z3 = third(z);
   unsigned r[ROW];
-  int at = far ? i + (BOYSYDF_NNEAR - 256) : i;
+  int at = far ? min(i, 1024) + (BOYSYDF_NNEAR - 256) : i;
   if (!HF_BCHECK(kc, at >= 0 && at < BOYSYDF_NNEAR + BOYSY_NFAR, HF_BC_BOYS, at)) at = 0;
   const unsigned* const row = kc.boysydf + boysydf_off(L) + (size_t)at * ROW;
 #pragma unroll

@@ -20,7 +20,8 @@ static inline float __fmul_rn(float a, float b) { return a * b; }
 static inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
 static inline float __double2float_rn(double x) { return (float)x; }
 static inline float rsqrtf(float x) { return 1.0f / std::sqrt(x); }
-static inline int __float2int_rn(float x) { return (int)std::nearbyint(x); }
+// the device's conversion saturates, and gives 0 for a NaN
+static inline int __float2int_rn(float x) { return x != x ? 0 : x >= 2147483648.0f ? 2147483647 : (int)std::nearbyint(x); }
 static inline int __double2hiint(double x) { return (int)(same_bits<long long>(x) >> 32); }
 static inline int __double2loint(double x) { return (int)same_bits<long long>(x); }
 static inline double __hiloint2double(int h, int l) { return same_bits<double>((long long)(((unsigned long long)(unsigned)h << 32) | (unsigned)l)); }
@@ -31,6 +32,7 @@ static inline float __uint_as_float(unsigned x) { return same_bits<float>(x); }
 static inline float __int_as_float(int x) { return same_bits<float>(x); }
 // the hardware's estimate: the low word is zero
 static inline double host_rsqrt_estimate(double a) { return same_bits<double>(same_bits<long long>(1.0 / std::sqrt(a)) & ~0xffffffffll); }
+static inline int min(int a, int b) { return a < b ? a : b; }
 #include "herm_host.cuh"
 
 // S_0 .. S_L at y in FP64 (s) and df64 (d: hi, lo pairs; y is split into a pair)

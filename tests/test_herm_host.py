@@ -17,6 +17,7 @@ import os
 import re
 import shutil
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -47,6 +48,7 @@ def lib(tmp_path_factory):
     subprocess.run([cxx, "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", d, "-I", CSRC, "-I", inc,
                     os.path.join(ROOT, "tests", "herm_host_harness.cpp"), "-o", out], check=True)
     h = ctypes.CDLL(out)
+    h.path = out
     h.t64, h.tdf = np.zeros(h.words64(), np.uint32), np.zeros(h.wordsdf(), np.uint32)
     tables._Z13hf_boysy_fillPjS_(h.t64.ctypes.data_as(ctypes.c_void_p), h.tdf.ctypes.data_as(ctypes.c_void_p))
     return h
@@ -104,3 +106,25 @@ def test_rsqrt_of_every_exponent(lib):
         for a in np.concatenate([np.exp(RNG.uniform(np.log(1e-30), np.log(1e30), 300)), [1.0, 2.0, 4.0, 0.25, np.nextafter(1.0, 0)]]):
             got = lib.rsqrt64(ctypes.c_double(float(a)))
             assert abs(mp.mpf(got) * mp.sqrt(mp.mpf(float(a))) - 1) <= 1.5 * 2.0 ** -53
+
+
+CHILD = """
+import ctypes, sys
+import numpy as np
+h, t = ctypes.CDLL(sys.argv[1]), np.load(sys.argv[2])
+p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+for L in range(9):
+    for y in (1e38, 3.5e38, 1e200, float("inf"), float("nan")):
+        s, d = np.zeros(L + 1), np.zeros(2 * L + 2, np.float32)
+        h.s_all(L, p(t["t64"]), p(t["tdf"]), ctypes.c_double(y), p(s), p(d))
+        assert y > 1e38 or np.all(np.abs(d[::2]) <= 2.0 ** -60), (L, y, d)
+print("ok")
+"""
+
+
+def test_arguments_beyond_the_range_of_floats_stay_in_the_tables(lib, tmp_path):
+    """Centres 1e16 bohr apart are accepted; y = 2T then overflows a float, and the row index with it.
+    In a child process: an index out of range ends it."""
+    np.savez(tmp_path / "t.npz", t64=lib.t64, tdf=lib.tdf)
+    r = subprocess.run([sys.executable, "-c", CHILD, lib.path, str(tmp_path / "t.npz")], capture_output=True, text=True)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stderr[-500:]
