@@ -3,6 +3,8 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "hf_internal.h"
@@ -103,8 +105,9 @@ static void boys_row(long double T, long double* F, long double* et) {
 }
 
 // Rows of the S_m(y) tables (hf_device.h): near rows from boys_row, far rows
-// from the large-T form F_m = sqrt(pi / T) / 2 (2m - 1)!! / (2T)^m.
-void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
+// from the large-T form F_m = sqrt(pi / T) / 2 (2m - 1)!! / (2T)^m.  Rows k, k +
+// n, ... of each kind, by one of n threads.
+static void boysy_rows(uint32_t* t64, uint32_t* tdf, int k, int n) {
   auto split = [](long double c, float* q) {
     q[0] = (float)c;
     q[1] = (float)(c - (long double)q[0]);
@@ -141,7 +144,7 @@ void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
       memcpy(r + 3 + m, &v, sizeof v);
     }
   };
-  for (int i = 0; i < BOYSYDF0_NNEAR; ++i) {
+  for (int i = k; i < BOYSYDF0_NNEAR; i += n) {
     boys_row((long double)i / 128.0L, F, &et);
     for (int m = 1; m < BOYS_NM; m += 2) F[m] = -F[m];
     row0(i);
@@ -149,7 +152,7 @@ void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
     if (i % 8 == 0) rows(tdf, i / 8, true);
   }
   const long double pi = 3.141592653589793238462643383279502884L;
-  for (int i = 0; i < BOYSYDF0_NFAR; ++i) {
+  for (int i = k; i < BOYSYDF0_NFAR; i += n) {
     const long double T = (1024 + i) / 64.0L;
     F[0] = 0.5L * sqrtl(pi / T);
     for (int m = 1; m < BOYS_NM; ++m) F[m] = -F[m - 1] * (2 * m - 1) / (2.0L * T);
@@ -159,11 +162,35 @@ void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
   }
 }
 
-int hf_boys_tables(hf_ctx* ctx) {
-  const size_t n64 = (size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS64_ROW;
-  const size_t n32 = (size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS32_ROW;
-  std::vector<double> t64(n64);
-  std::vector<float> t32(n32);
+// long double is a software type on Arm hosts: 73 ms by one thread there.
+void hf_boysy_fill(uint32_t* t64, uint32_t* tdf) {
+  constexpr int kThreads = 8;
+  std::vector<std::thread> th;
+  int started = 1;  // part 0 is the caller's
+  try {
+    th.reserve(kThreads);
+    for (; started < kThreads; ++started) th.emplace_back(boysy_rows, t64, tdf, started, kThreads);
+  } catch (...) {  // no thread to be had: the caller does the rest
+  }
+  boysy_rows(t64, tdf, 0, kThreads);
+  for (int k = started; k < kThreads; ++k) boysy_rows(t64, tdf, k, kThreads);
+  for (std::thread& t : th) t.join();
+}
+
+// The tables on the host, computed once per process (every context uploads them).
+namespace {
+struct BoysHost {
+  std::vector<double> t64;
+  std::vector<float> t32, tdf;
+  std::vector<uint32_t> y64, ydf, coop;
+  BoysHost();
+};
+}  // namespace
+
+BoysHost::BoysHost()
+    : t64((size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS64_ROW), t32((size_t)(BOYS_LMAX + 1) * BOYS_NGRID * BOYS32_ROW),
+      tdf((size_t)(BOYS_LMAX + 1) * BOYSDF_NGRID * BOYSDF_ROW, 0.0f), y64(boysy64_off(BOYSY_LMAX + 1), 0u),
+      ydf(boysydf_off(BOYSY_LMAX + 1), 0u), coop(hf_coop_tables()) {
   long double F[BOYS_NM], et;
   long double fact[BOYS64_TERMS];
   fact[0] = 1.0L;
@@ -186,8 +213,6 @@ int hf_boys_tables(hf_ctx* ctx) {
   // df64 table: grid T_i = i/16, per (order, row) 16 floats: the Taylor
   // coefficients of F_L (c_0..c_4 as hi/lo pairs, c_5..c_7 as floats), a pad,
   // and exp(-T_i) as a hi/lo pair
-  const size_t ndf = (size_t)(BOYS_LMAX + 1) * BOYSDF_NGRID * BOYSDF_ROW;
-  std::vector<float> tdf(ndf, 0.0f);
   auto split = [](long double c, float* q) {
     const float h = (float)c;
     q[0] = h;
@@ -206,28 +231,25 @@ int hf_boys_tables(hf_ctx* ctx) {
     }
   }
   // S_m(y) = (-1)^m F_m(y / 2) of the Hermite kernels (layout in hf_device.h)
-  std::vector<uint32_t> ty(boysy64_off(BOYSY_LMAX + 1), 0u), tyd(boysydf_off(BOYSY_LMAX + 1), 0u);
-  hf_boysy_fill(ty.data(), tyd.data());
-  void* p = nullptr;
-  HF_CHECK(hf_dev_alloc(ctx, &p, ty.size() * sizeof(uint32_t)));
-  ctx->boysy64 = (uint32_t*)p;
-  HF_CUDA(cudaMemcpyAsync(ctx->boysy64, ty.data(), ty.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-  HF_CHECK(hf_dev_alloc(ctx, &p, tyd.size() * sizeof(uint32_t)));
-  ctx->boysydf = (uint32_t*)p;
-  HF_CUDA(cudaMemcpyAsync(ctx->boysydf, tyd.data(), tyd.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-  const std::vector<uint32_t> ct = hf_coop_tables();
-  HF_CHECK(hf_dev_alloc(ctx, &p, ct.size() * sizeof(uint32_t)));
-  ctx->cooptab = (uint32_t*)p;
-  HF_CUDA(cudaMemcpyAsync(ctx->cooptab, ct.data(), ct.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-  HF_CHECK(hf_dev_alloc(ctx, &p, ndf * sizeof(float)));
-  ctx->boysdf = (float*)p;
-  HF_CUDA(cudaMemcpyAsync(ctx->boysdf, tdf.data(), ndf * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-  HF_CHECK(hf_dev_alloc(ctx, &p, n64 * sizeof(double)));
-  ctx->boys64 = (double*)p;
-  HF_CHECK(hf_dev_alloc(ctx, &p, n32 * sizeof(float)));
-  ctx->boys32 = (float*)p;
-  HF_CUDA(cudaMemcpyAsync(ctx->boys64, t64.data(), n64 * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-  HF_CUDA(cudaMemcpyAsync(ctx->boys32, t32.data(), n32 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+  hf_boysy_fill(y64.data(), ydf.data());
+}
+
+int hf_boys_tables(hf_ctx* ctx) {
+  static const BoysHost h;
+  auto up = [&](auto** dst, const auto& v) {
+    const size_t bytes = v.size() * sizeof(v[0]);
+    void* p = nullptr;
+    HF_CHECK(hf_dev_alloc(ctx, &p, bytes));
+    *dst = static_cast<std::remove_reference_t<decltype(**dst)>*>(p);
+    HF_CUDA(cudaMemcpyAsync(p, v.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
+    return (int)HF_OK;
+  };
+  HF_CHECK(up(&ctx->boysy64, h.y64));
+  HF_CHECK(up(&ctx->boysydf, h.ydf));
+  HF_CHECK(up(&ctx->cooptab, h.coop));
+  HF_CHECK(up(&ctx->boysdf, h.tdf));
+  HF_CHECK(up(&ctx->boys64, h.t64));
+  HF_CHECK(up(&ctx->boys32, h.t32));
   HF_CUDA(cudaStreamSynchronize(ctx->stream));
   return HF_OK;
 }
