@@ -192,28 +192,26 @@ __global__ void __launch_bounds__(kThreads) eig_kernel(const EigBatch batch) {
     for (int t = tid; t < n * n; t += kThreads) job.A[t] = nan("");
     for (int i = tid; i < n; i += kThreads) job.w[i] = nan("");
   };
-  // largest element
+  // largest element, infinite if one is not finite (tests and powers of two on
+  // the exponent bits: a solve waits for every FP64 instruction here)
+  auto expo = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
   double mx = 0.0;
-  int bad = 0;
   for (int t = tid; t < n * n; t += kThreads) {
-    const int j = t / n, i = t - j * n;
-    if (i < j) continue;
-    const double v = fabs(A[t]);
-    bad |= !(v <= 1.7976931348623157e308);
-    mx = fmax(mx, v);
-  }
-  if (__syncthreads_or(bad)) {
-    no_result();
-    return;
+    const double v = A[t];
+    mx = expo(v) == 0x7ff ? INFINITY : fmax(mx, fabs(v));
   }
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((tid & 31) == 0) red[tid >> 5] = mx;
   __syncthreads();
   mx = red[0];
   for (int k = 1; k < kThreads / 32; ++k) mx = fmax(mx, red[k]);
-  // scaled by a power of two (exactly) to elements in [-1, 1] ([-2, 2] at the end of the range)
-  const int ex = mx > 0.0 ? max(-1022, min(1023, ilogb(mx) + 1)) : 0;
-  const double down = scalbn(1.0, -ex), up = scalbn(1.0, ex);
+  if (expo(mx) == 0x7ff) {  // the same in every thread
+    no_result();
+    return;
+  }
+  // scaled by a power of two (exactly) to elements in [-1, 1], a little above at the ends of the range
+  const int ex = mx > 0.0 ? max(-1022, min(1022, expo(mx) - 1022)) : 0;
+  const double down = __hiloint2double((1023 - ex) << 20, 0), up = __hiloint2double((1023 + ex) << 20, 0);
   auto el = [&](int i, int j) -> double {
     return i < n && j < n ? A[(size_t)min(i, j) * n + max(i, j)] * down : 0.0;
   };
