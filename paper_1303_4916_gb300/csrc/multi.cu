@@ -255,12 +255,10 @@ int MultiJK::capture(const KernelCommon& kc) {
     cudaGraphDestroy(graph);
     graph = nullptr;
   }
-  // make sure the occupancy queries are answered outside the capture
+  // make sure the occupancy queries of the launches are answered outside the capture
   for (int c = 0; c < HF_NCLASS; ++c) {
-    ctx->ops[c].occ64();
-    ctx->ops[c].occ32();
-    ctx->ops[c].occdf();
-    ctx->ops[c].occrys();
+    if (w[2 * c].nitems > 0) hf_occ_hi(ctx->ops[c], jk_flags);
+    if (w[2 * c + 1].nitems > 0) hf_occ_lo(ctx->ops[c], jk_flags);
   }
   HF_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   capturing = true;
