@@ -10,7 +10,7 @@
 // ket's coefficients once per group.  The Obara-Saika node lists this replaces
 // evaluated every node of the bra and of the ket per primitive quartet
 // (a J/K build of a 9-atom s+p+d molecule 22.7 -> 20.2 ms in FP64, of a 20-atom
-// one in df64 with an FP32 split 45 -> 36.4 ms).
+// one in df64 with an FP32 split 45 -> 36.4 ms, 36.6 with the range rule below).
 // Index tables (coop_tab.cu) are kept with the context.
 //
 // Range in df64: the set-up forms w^m, m <= 8, w = 2 rho up to twice the smaller
