@@ -56,3 +56,21 @@ def test_tensor_repeats_to_the_last_bit(hf, ctx, case):
         assert torch.equal(G.permute(*p), G)
     G0 = oracle.Basis(mol).eri_tensor()
     assert np.max(np.abs(G.cpu().numpy() - G0)) <= 1e-12 * max(1.0, np.max(np.abs(G0)))
+
+
+def test_tensor_of_a_class_too_large_for_slots(hf, ctx):
+    """34 p shells of 5 primitives: the (pp|pp) quartets' unit slots would pass 256 MB, so the class takes whole kets.
+    J and K from the tensor against the direct build, which has lists of its own."""
+    import torch
+    rng = np.random.default_rng(8)
+    n = 34
+    xyz = np.array([[i % 4, i // 4 % 3, i // 12] for i in range(n)]) * 1.3 + rng.uniform(-0.1, 0.1, (n, 3))
+    shells = [(a, 1, np.exp(rng.uniform(np.log(0.3), np.log(3.0), 5)), rng.uniform(0.2, 1.0, 5)) for a in range(n)]
+    b = hf.Basis(ctx, _pack([1] * n, xyz, shells, "p34", -1))
+    G = b.eri_tensor()
+    assert torch.equal(b.eri_tensor(), G)
+    C = rng.normal(size=(b.nbf, 10)) / np.sqrt(b.nbf)
+    D = torch.tensor(C @ C.T, device="cuda:0")
+    J, K = b.jk_stored(G, D)
+    J0, K0 = b.fock_jk(D, opts=hf.jk_opts(0.0))
+    assert float((J - J0).abs().max()) <= 1e-10 and float((K - K0).abs().max()) <= 1e-10

@@ -20,7 +20,8 @@ def lib(tmp_path):
     if not cxx or not os.path.isdir(inc):
         pytest.skip("no host C++ compiler or CUDA headers")
     out = str(tmp_path / "libpd.so")
-    subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-I", inc,
+    # -Bsymbolic: the fake runtime answers also where a real libcudart is in the process
+    subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CSRC, "-I", inc,
                     os.path.join(ROOT, "tests", "per_device_harness.cpp"), "-o", out], check=True)
     return ctypes.CDLL(out)
 
